@@ -473,6 +473,7 @@ size_t carve(ibm_state* s, void* base, const Layout& L, Fields<T>& f) {
   fl.slot = cv.take<double>(3 * (size_t)L.nslot);
   fl.csr_off = cv.take<int>(L.nf + 1);
   fl.csr_idx = cv.take<int>(L.ncsr);
+  fl.lat = cv.take<float4>(4 * (size_t)L.nf);
   s->prm = f.prm;
   if (s->precision == IBM_MIXED) {
     s->hy = cv.take<float>((size_t)c.ny * c.ny);
@@ -650,6 +651,41 @@ void record_graph(ibm_state* s, int kind, int cur) {
   if (join) cudaStreamWaitEvent(s->stream, s->ev_join, 0);
 }
 
+// data of the lattice form of the structural update (k_flag_patch): lengths are
+// scaled by the power of two that brings the longest rest length into
+// [1/2, 1), so its FP32 pairs stay near 1 whatever the flag's size
+std::vector<float4> lattice_rest(const FlagGeom& g, const ibm_bodies& b, Flag& fl) {
+  auto pair = [](double v) {
+    const float h = (float)v;
+    return make_float2(h, (float)(v - (double)h));
+  };
+  const int ns = g.ns, nt = g.nt;
+  double longest = 0.0;
+  for (double l : g.l0) longest = std::max(longest, l);
+  int e = 0;
+  std::frexp(longest, &e);
+  const double scale = std::ldexp(1.0, -e);
+  std::vector<float4> lat(4 * (size_t)ns * nt, make_float4(1.0f, 0.0f, 1.0f, 0.0f));
+  for (size_t q = 0; q < g.l0.size(); ++q) {
+    const int p = g.spring[2 * q], r = g.spring[2 * q + 1];
+    const int da = r / nt - p / nt, dc = r % nt - p % nt;
+    // S (1, 0), T (0, 1), D (1, 1); E runs from v10 to v01 (-1, 1), its cell is one row below p
+    const int kind = da == 0 ? 1 : da < 0 ? 3 : dc == 0 ? 0 : 2;
+    const int point = kind == 3 ? p - nt : p;
+    const float2 l = pair(g.l0[q] * scale), l2 = pair(g.l0[q] * scale * (g.l0[q] * scale));
+    lat[4 * (size_t)point + kind] = make_float4(l.x, l.y, l2.x, l2.y);
+  }
+  const double ds = b.flag_len / (ns - 1), dt = b.flag_span / (nt - 1), cell = ds * dt;
+  fl.k_edge[0] = pair(0.5 * (b.bending * (ds * ds) / cell));
+  fl.k_edge[1] = pair(0.5 * (b.bending * (dt * dt) / cell));
+  fl.k_edge[2] = pair(0.5 * (2.0 * b.bending * cell / (ds * ds + dt * dt)));
+  fl.k_edge[3] = pair(b.stretch / (scale * scale));
+  fl.force_scale = scale;
+  fl.fix_scale = std::ldexp(scale, 49);
+  for (int q = 0; q < 3; ++q) fl.fix_x0[q] = g.X[q] * fl.fix_scale;
+  return lat;
+}
+
 template <class T>
 int init_state(ibm_state* s, const ibm_options* o, const FlagGeom& fg,
                const std::vector<double>& Xb, double bar_dv, const BarMask& bm) {
@@ -714,12 +750,16 @@ int init_state(ibm_state* s, const ibm_options* o, const FlagGeom& fg,
     CK(up(fl.tri_k, fg.tri_k.data(), fg.tri_k.size() * sizeof(double)));
     CK(up(fl.csr_off, fg.csr_off.data(), fg.csr_off.size() * sizeof(int)));
     CK(up(fl.csr_idx, fg.csr_idx.data(), fg.csr_idx.size() * sizeof(int)));
+    const std::vector<float4> lat = lattice_rest(fg, s->bodies, fl);
+    CK(up(fl.lat, lat.data(), lat.size() * sizeof(float4)));
+    CK(cudaStreamSynchronize(st));
     // enough CTAs for the hinge work, within the cluster limit
     const int want = std::min((fl.n_tri + fl.n_spring + 1023) / 1024, flag_max_cluster());
     fl.cluster = 1;
     while (2 * fl.cluster <= want) fl.cluster *= 2;
     // the structural update runs beside the pressure solve: persistent
     // kernels there leave its SMs free instead of queueing behind it
+    if (flag_patches(fl.ns, fl.nt, &fl.patch_r, &fl.patch_c)) fl.cluster = fl.patch_r * fl.patch_c;
     s->c.sm_reserved = fl.cluster;
   }
   // parameters

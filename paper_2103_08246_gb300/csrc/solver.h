@@ -83,6 +83,15 @@ struct Flag {
   int* csr_off = nullptr;     // nv + 1 offsets into csr_idx
   int* csr_idx = nullptr;     // slot ids contributing to each vertex
   int cluster = 1;            // CTAs cooperating in the structure kernel
+  // lattice form (k_flag_patch): the cluster's patches along s and t (0: not
+  // used), rest data of the springs S, T, D, E of every lattice point (scaled
+  // length and its square, each an FP32 pair), hinge stiffnesses across S, T and
+  // diagonal edges and the scaled spring constant (FP32 pairs), and the powers
+  // of two of the scaled lattice
+  int patch_r = 0, patch_c = 0;
+  float4* lat = nullptr;
+  float2 k_edge[4] = {};
+  double fix_scale = 0.0, fix_x0[3] = {0.0, 0.0, 0.0}, force_scale = 0.0;
 };
 
 // one case of a batched explicit stage: its constants, step parameters,
@@ -210,5 +219,7 @@ void slab_unpack_force(const Consts& c, Params* prm, const Flag& fl, const doubl
 void launch_flag(Params* prm, const Flag& fl, bool force, cudaStream_t s);
 void launch_flag_stats(const Flag& fl, double* out, cudaStream_t s);
 int flag_max_cluster();
+// patches of an ns x nt lattice for k_flag_patch; false: the list form
+bool flag_patches(int ns, int nt, int* pr, int* pc);
 
 }  // namespace ibm
