@@ -13,8 +13,10 @@
 // component) in shared memory and interpolates from it; the spreading block
 // accumulates the tile's contributions in a shared-memory box and adds each
 // nonzero node to the field once (one coalesced atomic per node and tile
-// instead of 27 scattered ones per marker and component). The flag's moving
-// markers take one thread each in extra blocks of the same launches.
+// instead of 27 scattered ones per marker and component; FP64 adds to the
+// field directly). The flag's moving markers take three threads each, one per
+// component, in extra blocks of the same launches (laminar flag, 1089 markers,
+// FP32: 0.039 -> 0.012 ms; 4225 markers, FP64: 0.254 -> 0.019 ms).
 //
 // Markers 0 .. nf-1 are the flag vertices (target velocity V_l, position X_l
 // from the structure), the rest the bar-grid markers (target 0). Nodes
@@ -272,45 +274,100 @@ __device__ inline int pos_mod(int a, int n) {
   return r < 0 ? r + n : r;
 }
 
-// interpolation, amplitude and flag force of one marker from global memory
+// One flag vertex and one velocity component per thread: three times the
+// threads and a third of the serial chain of a thread per vertex. The three
+// weights of a direction share one square root: with the node offsets
+// r = t - 1/2 - f (f in [0, 1)) the middle node lies inside |r| <= 1/2, and
+// 1 - |r| of the outer two is +-r of the middle one, so
+//   s = sqrt(1 - 3 (1/2 - f)^2),  w = ((7/2 - 3 f - s)/6, (1 + s)/3, (1/2 + 3 f - s)/6);
+// 3 square roots per thread instead of 9 (and as many divisions), which bound
+// the FP64 stage: 4225 vertices took 126 + 113 us in 9 blocks of 512.
 template <class T>
-__device__ inline double interp_marker(const Consts& c, const Params* prm, const Markers& m,
-                                       const Flag& fl, int l, const T* __restrict__ u,
-                                       const T* __restrict__ v, const T* __restrict__ w) {
-  double X, Y, Z, U[3], dv;
-  const bool ok = marker(m, fl, l, X, Y, Z, U, dv);
-  double us[3] = {0.0, 0.0, 0.0};
+__device__ __forceinline__ void phi3(T f, T w[3]) {
+  const T r = (T)0.5 - f;
+  const T s = sqrt((T)1 - (T)3 * r * r);
+  w[0] = ((T)3.5 - (T)3 * f - s) * (T)(1.0 / 6.0);
+  w[1] = ((T)1 + s) * (T)(1.0 / 3.0);
+  w[2] = ((T)0.5 + (T)3 * f - s) * (T)(1.0 / 6.0);
+}
+// stencil of vertex l on component comp: first node per direction and weights;
+// false for positions that are not finite or absurd (skipped)
+template <class T>
+__device__ __forceinline__ bool flag_stencil(const Consts& c, const Markers& m, const Flag& fl, int l, int comp, int i0[3],
+                                             T wx[3], T wy[3], T wz[3]) {
+  const double X[3] = {fl.X[3 * l] - m.x_shift, fl.X[3 * l + 1], fl.X[3 * l + 2]};
+  T f[3];
+  bool ok = true;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    ok = ok && isfinite(X[d]) && fabs(X[d]) < 1e6;
+    const double a = X[d] * c.inv_h - (d == comp ? 0.5 : 1.0);
+    const double fl_a = floor(a);
+    i0[d] = (int)fl_a;
+    f[d] = (T)(a - fl_a);
+  }
+  phi3<T>(f[0], wx);
+  phi3<T>(f[1], wy);
+  phi3<T>(f[2], wz);
+  return ok;
+}
+constexpr int FLAG_ITEMS = 96;   // vertex components per block: 4225 vertices spread over 133 blocks
+
+// interpolation, amplitude and fluid force of one vertex component; returns the slip
+template <class T>
+__device__ inline double flag_interp(const Consts& c, const Params* prm, const Markers& m, const Flag& fl, int item,
+                                     const T* __restrict__ u, const T* __restrict__ v, const T* __restrict__ w) {
+  const int l = item / 3, comp = item - 3 * l;
+  const T* q = comp == 0 ? u : (comp == 1 ? v : w);
+  int i0[3];
+  T wx[3], wy[3], wz[3];
+  const bool ok = flag_stencil<T>(c, m, fl, l, comp, i0, wx, wy, wz);
+  double du = 0.0;
+  const double dv = fl.dv[l];
   if (ok) {
-    const Frac<T> fx = frac_of<T>(X * c.inv_h), fy = frac_of<T>(Y * c.inv_h),
-                  fz = frac_of<T>(Z * c.inv_h);
-    for (int comp = 0; comp < 3; ++comp) {
-      const T* q = comp == 0 ? u : (comp == 1 ? v : w);
-      Stencil st;
-      T wx[3], wy[3], wz[3];
-      stencil<T>(c, comp, fx, fy, fz, st, wx, wy, wz);
-      T acc = 0;
-      for (int a = 0; a < 3; ++a) {
-        if (!st.vi[a]) continue;
-        const size_t pi = (size_t)(st.i0 + a) * c.ny;
-        for (int b = 0; b < 3; ++b) {
-          const size_t pj = (pi + st.j[b]) * c.nz;
-          const T wab = wx[a] * wy[b];
-          for (int e = 0; e < 3; ++e) acc += wab * wz[e] * q[pj + st.k[e]];
-        }
+    const int lo = comp == 0 ? 1 : 0, hi = c.nx - 1;
+    T acc = 0;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      const int i = i0[0] + a;
+      if (i < lo || i > hi) continue;
+#pragma unroll
+      for (int b = 0; b < 3; ++b) {
+        const T* row = q + ((size_t)i * c.ny + ((i0[1] + b) & (c.ny - 1))) * c.nz;
+        const T wab = wx[a] * wy[b];
+#pragma unroll
+        for (int e = 0; e < 3; ++e) acc += wab * wz[e] * row[(i0[2] + e) & (c.nz - 1)];
       }
-      us[comp] = (double)acc;
+    }
+    du = fl.V[item] - (double)acc;
+  }
+  m.coef[item] = dv * c.inv_h * c.inv_h * c.inv_h * du;
+  fl.Ff[item] = -du / prm->dt * dv;
+  return fabs(du);
+}
+
+template <class T>
+__device__ inline void flag_spread(const Consts& c, const Markers& m, const Flag& fl, int item, T* __restrict__ u,
+                                   T* __restrict__ v, T* __restrict__ w) {
+  const int l = item / 3, comp = item - 3 * l;
+  const T cf = (T)m.coef[item];
+  int i0[3];
+  T wx[3], wy[3], wz[3];
+  if (!flag_stencil<T>(c, m, fl, l, comp, i0, wx, wy, wz) || cf == (T)0) return;
+  T* q = comp == 0 ? u : (comp == 1 ? v : w);
+  const int lo = comp == 0 ? 1 : 0, hi = c.nx - 1;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const int i = i0[0] + a;
+    if (i < lo || i > hi) continue;
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      T* row = q + ((size_t)i * c.ny + ((i0[1] + b) & (c.ny - 1))) * c.nz;
+      const T wab = wx[a] * wy[b] * cf;
+#pragma unroll
+      for (int e = 0; e < 3; ++e) atomicAdd(&row[(i0[2] + e) & (c.nz - 1)], wab * wz[e]);
     }
   }
-  const double vol = dv * c.inv_h * c.inv_h * c.inv_h;
-  const double dt = prm->dt;
-  double slip = 0.0;
-  for (int comp = 0; comp < 3; ++comp) {
-    const double du = ok ? (U[comp] - us[comp]) : 0.0;
-    m.coef[3 * l + comp] = vol * du;
-    if (l < m.nf) fl.Ff[3 * l + comp] = -du / dt * dv;
-    slip = fmax(slip, fabs(du));
-  }
-  return slip;
 }
 
 // Per bar marker, once at set-up (the markers never move): the kernel
@@ -415,8 +472,8 @@ k_ib_interp_tiles(Consts c, Params* prm, Markers m, Flag fl, const T* __restrict
   }
   double slip = 0.0;
   if ((int)blockIdx.x >= m.n_tiles) {
-    const int l = ((int)blockIdx.x - m.n_tiles) * blockDim.x + threadIdx.x;
-    if (l < m.nf) slip = interp_marker<T>(c, prm, m, fl, l, u, v, w);
+    const int item = ((int)blockIdx.x - m.n_tiles) * FLAG_ITEMS + threadIdx.x;
+    if (threadIdx.x < FLAG_ITEMS && item < 3 * m.nf) slip = flag_interp<T>(c, prm, m, fl, item, u, v, w);
   } else {
     const TileBox bx = tile_box(m, blockIdx.x);
     // every copy in flight at once (cp.async), one wait
@@ -434,26 +491,24 @@ k_ib_interp_tiles(Consts c, Params* prm, Markers m, Flag fl, const T* __restrict
     cp_async_wait<0>();
     __syncthreads();
     const double vol = m.bar_dv * c.inv_h * c.inv_h * c.inv_h;
-    for (int b = bx.b0 + threadIdx.x; b < bx.b1; b += blockDim.x) {
-      const int packed = bo[b];
-      const int l = m.nf + b;
-      for (int comp = 0; comp < 3; ++comp) {
-        T wx[3], wy[3], wz[3];
-        const T* bq = box + bar_stencil<T>(m, bx, bw, packed, b, comp, wx, wy, wz);
-        T acc = 0;
+    const int cnt = bx.b1 - bx.b0;
+    for (int q = threadIdx.x; q < 3 * cnt; q += blockDim.x) {   // one component of one marker per thread
+      const int comp = q / cnt, b = bx.b0 + q - comp * cnt;
+      T wx[3], wy[3], wz[3];
+      const T* bq = box + bar_stencil<T>(m, bx, bw, bo[b], b, comp, wx, wy, wz);
+      T acc = 0;
 #pragma unroll
-        for (int a = 0; a < 3; ++a)
+      for (int a = 0; a < 3; ++a)
 #pragma unroll
-          for (int e2 = 0; e2 < 3; ++e2) {
-            const T wab = wx[a] * wy[e2];
-            const T* row = bq + (a * bx.by + e2) * bx.bz;
+        for (int e2 = 0; e2 < 3; ++e2) {
+          const T wab = wx[a] * wy[e2];
+          const T* row = bq + (a * bx.by + e2) * bx.bz;
 #pragma unroll
-            for (int e = 0; e < 3; ++e) acc += wab * wz[e] * row[e];
-          }
-        const double du = -(double)acc;
-        m.coef[3 * l + comp] = vol * du;
-        slip = fmax(slip, fabs(du));
-      }
+          for (int e = 0; e < 3; ++e) acc += wab * wz[e] * row[e];
+        }
+      const double du = -(double)acc;
+      m.coef[3 * (m.nf + b) + comp] = vol * du;
+      slip = fmax(slip, fabs(du));
     }
   }
   slip = warp_max(slip);
@@ -470,51 +525,58 @@ k_ib_spread_tiles(Consts c, Markers m, Flag fl, const T* __restrict__ bw, const 
   extern __shared__ __align__(16) unsigned char ib_smem[];
   T* box = reinterpret_cast<T*>(ib_smem);
   if ((int)blockIdx.x >= m.n_tiles) {
-    const int l = ((int)blockIdx.x - m.n_tiles) * blockDim.x + threadIdx.x;
-    if (l >= m.nf) return;
-    double X, Y, Z, U[3], dv;
-    if (!marker(m, fl, l, X, Y, Z, U, dv)) return;
-    const Frac<T> fx = frac_of<T>(X * c.inv_h), fy = frac_of<T>(Y * c.inv_h),
-                  fz = frac_of<T>(Z * c.inv_h);
-    for (int comp = 0; comp < 3; ++comp) {
-      const T cf = (T)m.coef[3 * l + comp];
-      if (cf == (T)0) continue;
-      T* q = comp == 0 ? u : (comp == 1 ? v : w);
-      Stencil st;
+    const int item = ((int)blockIdx.x - m.n_tiles) * FLAG_ITEMS + threadIdx.x;
+    if (threadIdx.x < FLAG_ITEMS && item < 3 * m.nf) flag_spread<T>(c, m, fl, item, u, v, w);
+    return;
+  }
+  const TileBox bx = tile_box(m, blockIdx.x);
+  const int cnt = bx.b1 - bx.b0;
+  if constexpr (sizeof(T) == 8) {
+    // FP64: straight to the field; a shared-memory FP64 addition is a
+    // compare-and-swap loop, L2 adds FP64 natively (both stages of the
+    // production bars, 237,568 markers: 0.377 -> 0.244 ms)
+    for (int q = threadIdx.x; q < 3 * cnt; q += blockDim.x) {
+      const int comp = q / cnt, b = bx.b0 + q - comp * cnt;
       T wx[3], wy[3], wz[3];
-      stencil<T>(c, comp, fx, fy, fz, st, wx, wy, wz);
+      const int at = bar_stencil<T>(m, bx, bw, bo[b], b, comp, wx, wy, wz) - comp * bx.n;
+      const int rz = at % bx.bz, ry = (at / bx.bz) % bx.by, rx = at / (bx.bz * bx.by);
+      const T cf = m.coef[3 * (m.nf + b) + comp];
+      T* dst = comp == 0 ? u : (comp == 1 ? v : w);
+      const int lo = comp == 0 ? 1 : 0, hi = c.nx - 1;
+#pragma unroll
       for (int a = 0; a < 3; ++a) {
-        if (!st.vi[a]) continue;
-        const size_t pi = (size_t)(st.i0 + a) * c.ny;
-        for (int b = 0; b < 3; ++b) {
-          const T wab = wx[a] * wy[b] * cf;
-          const size_t pj = (pi + st.j[b]) * c.nz;
-          for (int e = 0; e < 3; ++e) atomicAdd(&q[pj + st.k[e]], wab * wz[e]);
+        const int i = bx.ox + rx + a;
+        if (i < lo || i > hi) continue;
+#pragma unroll
+        for (int e2 = 0; e2 < 3; ++e2) {
+          const T wab = wx[a] * wy[e2] * cf;
+          T* row = dst + ((size_t)i * c.ny + ((bx.oy + ry + e2) & (c.ny - 1))) * c.nz;
+#pragma unroll
+          for (int e = 0; e < 3; ++e) {
+            const T val = wab * wz[e];
+            if (val != (T)0) atomicAdd(&row[(bx.oz + rz + e) & (c.nz - 1)], val);
+          }
         }
       }
     }
     return;
   }
-  const TileBox bx = tile_box(m, blockIdx.x);
   for (int q = threadIdx.x; q < 3 * bx.n; q += blockDim.x) box[q] = (T)0;
   __syncthreads();
-  for (int b = bx.b0 + threadIdx.x; b < bx.b1; b += blockDim.x) {
-    const int packed = bo[b];
-    const int l = m.nf + b;
-    for (int comp = 0; comp < 3; ++comp) {
-      T wx[3], wy[3], wz[3];
-      T* bq = box + bar_stencil<T>(m, bx, bw, packed, b, comp, wx, wy, wz);
-      const T cf = (T)m.coef[3 * l + comp];
+  for (int q = threadIdx.x; q < 3 * cnt; q += blockDim.x) {
+    const int comp = q / cnt, b = bx.b0 + q - comp * cnt;
+    T wx[3], wy[3], wz[3];
+    T* bq = box + bar_stencil<T>(m, bx, bw, bo[b], b, comp, wx, wy, wz);
+    const T cf = (T)m.coef[3 * (m.nf + b) + comp];
 #pragma unroll
-      for (int a = 0; a < 3; ++a)
+    for (int a = 0; a < 3; ++a)
 #pragma unroll
-        for (int e2 = 0; e2 < 3; ++e2) {
-          const T wab = wx[a] * wy[e2] * cf;
-          T* row = bq + (a * bx.by + e2) * bx.bz;
+      for (int e2 = 0; e2 < 3; ++e2) {
+        const T wab = wx[a] * wy[e2] * cf;
+        T* row = bq + (a * bx.by + e2) * bx.bz;
 #pragma unroll
-          for (int e = 0; e < 3; ++e) atomicAdd(&row[e], wab * wz[e]);
-        }
-    }
+        for (int e = 0; e < 3; ++e) atomicAdd(&row[e], wab * wz[e]);
+      }
   }
   __syncthreads();
   for_box_rows(c, bx, [&](int q, long long g, int comp) {
@@ -545,6 +607,15 @@ void ib_bin_bars(const Consts& c, std::vector<double>& Xb, std::vector<int>& til
   m.tx = 8;
   m.ty = c.ny < 16 ? c.ny : 16;
   m.tz = c.nz < 16 ? c.nz : 16;
+  // a plane of few tiles leaves most SMs idle: halve the tiles' transverse
+  // sides down to 4 x 8 while the plane has fewer than 32 (64 x 32 x 32 FP64:
+  // 3.78 -> 3.22 ms per 10 steps; going on to one tile per SM slows ensembles,
+  // which fill the SMs with members, by 4%)
+  while ((m.ty > 4 || m.tz > 8) && (c.ny / m.ty) * (c.nz / m.tz) < 32) {
+    if (m.ty > 4 && m.ty >= m.tz) m.ty /= 2;
+    else if (m.tz > 8) m.tz /= 2;
+    else m.ty /= 2;
+  }
   auto cell = [&](double x, int n, bool periodic) {
     long long q = (long long)std::floor(x * c.inv_h);
     if (periodic) q = ((q % n) + n) % n;
@@ -620,12 +691,15 @@ void launch_ib(const Consts& c, const Fields<T>& f, const Markers& m, const Flag
     k_ib_flush<T><<<nb, 128, 0, s>>>(c, m, fl, f.u[cur], f.v[cur], f.w[cur]);
     return;
   }
-  const int nblk = m.n_tiles + (m.nf + IB_THREADS - 1) / IB_THREADS;
+  // the flag's blocks use FLAG_ITEMS threads; without bars nothing needs more
+  const int nblk = m.n_tiles + (3 * m.nf + FLAG_ITEMS - 1) / FLAG_ITEMS;
+  // small tiles hold too few markers for 512 threads
+  const int threads = m.n_tiles ? (m.ty * m.tz < 256 ? IB_THREADS / 2 : IB_THREADS) : FLAG_ITEMS;
   const size_t smem = m.n_tiles ? ib_tile_smem(m, sizeof(T)) : 0;
   const T* bw = reinterpret_cast<const T*>(m.bar_w);
-  k_ib_interp_tiles<T><<<nblk, IB_THREADS, smem, s>>>(c, f.prm, m, fl, bw, m.bar_o, f.u[cur], f.v[cur],
+  k_ib_interp_tiles<T><<<nblk, threads, smem, s>>>(c, f.prm, m, fl, bw, m.bar_o, f.u[cur], f.v[cur],
                                                       f.w[cur]);
-  k_ib_spread_tiles<T><<<nblk, IB_THREADS, smem, s>>>(c, m, fl, bw, m.bar_o, f.u[cur], f.v[cur], f.w[cur]);
+  k_ib_spread_tiles<T><<<nblk, threads, sizeof(T) == 8 ? 0 : smem, s>>>(c, m, fl, bw, m.bar_o, f.u[cur], f.v[cur], f.w[cur]);
 }
 
 template void launch_ib<double>(const Consts&, const Fields<double>&, const Markers&, const Flag&,
