@@ -152,7 +152,7 @@ typedef struct {
   const double* init_v;
   const double* init_w;
   /* Tile parameters (0: defaults). rhs_planes: x planes per block of the
-   * streamed explicit stage [16], in [2, 256]; afx_planes: x planes per
+   * streamed explicit stage [chosen from the grid], in [2, 256]; afx_planes: x planes per
    * segment of the implicit x factor [64]: 16 or 24 hold a segment in each
    * thread's registers; otherwise values up to 40 select 32-plane and larger
    * values 64-plane segments staged in shared memory (range [8, 256]);

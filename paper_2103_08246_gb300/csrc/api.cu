@@ -342,6 +342,7 @@ struct ibm_state {
   Fields<double> fd{};
   Fields<float> ff{};
   Markers mk{};
+  std::vector<int> bar_order;   // place of each bar marker in the reported order (empty: its own)
   Flag fl{};
   Params* prm = nullptr;
   double* dstat = nullptr;    // 16 doubles of device scratch for diagnostics
@@ -894,7 +895,7 @@ int prepare(const ibm_grid* g, const ibm_domain* d, const ibm_bodies* b, const i
   c.u_in = 1.0;
   c.f_inv_h = (float)c.inv_h;
   c.f_inv_h2 = (float)(c.inv_h * c.inv_h);
-  c.rhs_planes = (o && o->rhs_planes > 0) ? o->rhs_planes : 16;
+  c.rhs_planes = o ? o->rhs_planes : 0;   // 0: from the grid (launch_rhs)
   c.rhs_stages = (o && o->rhs_stages > 0) ? o->rhs_stages : 8;
   c.afx_planes = (o && o->afx_planes > 0) ? o->afx_planes : 64;
   c.mixed_tc = o ? o->mixed_tc_predictor : 0;
@@ -925,7 +926,7 @@ int prepare(const ibm_grid* g, const ibm_domain* d, const ibm_bodies* b, const i
     s->dom.lx = c.lx;
     s->mk.x_shift = xs;
   }
-  ib_bin_bars(c, Xb, bm.tiles, s->mk);
+  ib_bin_bars(c, Xb, bm.tiles, s->mk, s->bar_order);
   L.ntile = s->mk.n_tiles;
   for (int q = 0; q < 3; ++q) L.nbm[q] = bm.n[q];
   c.omega_max = fg.omega_max;
@@ -1796,6 +1797,16 @@ int ibm_get_markers(ibm_state* s, double* X, size_t n) {
     CK(cudaMemcpyAsync(X + 3 * (size_t)s->mk.nf, s->mk.Xb, 3 * (size_t)s->mk.nb * sizeof(double),
                        cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
+  if (!s->bar_order.empty()) {   // stored by smaller tiles than reported
+    try {
+      double* xb = X + 3 * (size_t)s->mk.nf;
+      const std::vector<double> stored(xb, xb + 3 * (size_t)s->mk.nb);
+      for (size_t b = 0; b < s->bar_order.size(); ++b)
+        std::copy_n(&stored[3 * b], 3, xb + 3 * (size_t)s->bar_order[b]);
+    } catch (const std::bad_alloc&) {
+      return IBM_ENOMEM;
+    }
+  }
   return IBM_OK;
 }
 

@@ -46,7 +46,7 @@ struct Consts {
   double h, inv_h, nu, lx, ly, lz;
   double u_in;        // inflow speed U
   double omega_max;   // structural stiffness bound (sub-step count)
-  int rhs_planes;     // tile: x planes per block of the streamed RHS
+  int rhs_planes;     // tile: x planes per block of the streamed RHS (0: chosen from the grid)
   int rhs_stages;     // tile: most x planes in the streamed RHS's ring
   int afx_planes;     // tile: x planes per block of the FP32 x factor
   int sm_reserved;    // SMs the structural update holds while the pressure solve runs

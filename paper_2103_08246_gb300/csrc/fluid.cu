@@ -38,12 +38,15 @@ __device__ inline double af_theta(double r) { return 2.0 * asinh(0.5 / sqrt(r));
 // patterns order like the values, so the maximum is taken on the integer
 // pipe. Each kernel writes only the fields it owns: the structural update
 // runs concurrently and owns flag_pending.
-__global__ void k_begin_step(Consts c, Params* prm, const double* __restrict__ partial,
+// The partials are cleared for the maxima that this step's projection adds.
+__global__ void k_begin_step(Consts c, Params* prm, double* __restrict__ partial,
                              int n_partial, double tol, int hmax) {
   __shared__ unsigned long long wmax[32];
   unsigned long long mb = 0ull;
-  for (int b = threadIdx.x; b < n_partial; b += blockDim.x)
+  for (int b = threadIdx.x; b < n_partial; b += blockDim.x) {
     mb = max(mb, (unsigned long long)__double_as_longlong(partial[b]));
+    partial[b] = 0.0;
+  }
   for (int o = 16; o > 0; o >>= 1) mb = max(mb, __shfl_xor_sync(0xffffffffu, mb, o));
   if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = mb;
   __syncthreads();
@@ -1567,31 +1570,63 @@ struct RunTile {
   static constexpr int E = 16 / sizeof(T);
   static constexpr int THREADS = 256;
 };
-// rows per block of the run kernels, 0 when the shape does not fit them
+// whether the grid fits the run kernels, and the grid of CFL partial maxima
+// (one per 256 threads and 16 planes, whatever the launch below)
+constexpr int PART_PLANES = 16;
 template <class T>
-int run_rows(const Consts& c) {
+int partial_rows(const Consts& c) {
   const int runs = c.nz / RunTile<T>::E;
   if (runs < 1 || runs > RunTile<T>::THREADS || RunTile<T>::THREADS % runs) return 0;
   const int tj = RunTile<T>::THREADS / runs;
   return c.ny % tj == 0 ? tj : 0;
 }
-constexpr int RUN_XCH = 16;   // x planes per block of the run kernels
+// fewest x planes per block of the run kernels: chunks re-read the planes
+// beside them, which a small grid hides behind launch and load latency
+static int least_planes(const Consts& c) {
+  const long long cells = (long long)c.nx * c.ny * c.nz;
+  return cells <= (1 << 18) ? 2 : cells <= (1 << 20) ? 4 : 8;
+}
+
+// launch shape of the run kernels: threads and rows per block, x planes per
+// block; rows = 0 when the grid does not fit them. Blocks of 64 threads (or one
+// row) retire and start unevenly enough to keep loads in flight at the plane
+// loop's end: projection of 512 x 256 x 256 FP32 0.194 -> 0.184 ms against 256
+// threads. A block re-reads phi and u next to its first plane, so planes are
+// taken in chunks of `most`, fewer where that leaves under four blocks per SM
+// (64 x 32 x 32 FP64, 16 -> 2 planes and 64 threads: 0.068 -> 0.008 ms). FP32
+// grids in between gain nothing alone (256 x 128 x 128: 0.030 ms either way)
+// and lose 1% in an ensemble to the planes read twice: 256 threads, 16 planes.
+struct RunShape {
+  int threads, rows, xch;
+};
+template <class T>
+RunShape run_shape(const Consts& c, int planes, int most) {
+  RunShape r{64, 0, most};
+  if (!partial_rows<T>(c)) return r;
+  const long long cells = (long long)c.nx * c.ny * c.nz;
+  if (sizeof(T) == 4 && cells > (1 << 18) && cells < (1 << 23)) r = {RunTile<T>::THREADS, 0, PART_PLANES};
+  const int runs = c.nz / RunTile<T>::E;
+  if (r.threads < runs) r.threads = runs;
+  r.rows = r.threads / runs;   // divides ny: it divides the rows of a partial
+  while (r.xch > least_planes(c) && r.xch < PART_PLANES && (long long)(c.ny / r.rows) * ((planes + r.xch - 1) / r.xch) < 4 * 152) r.xch /= 2;
+  return r;
+}
 
 template <class T>
 __global__ void __launch_bounds__(256)
 k_div_vec(Consts c, const Params* __restrict__ prm, T* __restrict__ u, const T* __restrict__ v,
-          const T* __restrict__ w, T* __restrict__ phi, int initial) {
+          const T* __restrict__ w, T* __restrict__ phi, int initial, int xch) {
   constexpr int E = RunTile<T>::E;
   const int nx = c.nx, ny = c.ny, nz = c.nz;
   const int runs = nz / E;
-  const int tj = RunTile<T>::THREADS / runs;
+  const int tj = blockDim.x / runs;
   const int r = threadIdx.x / runs, k0 = (threadIdx.x - r * runs) * E;
   const int j = blockIdx.x * tj + r;
   const int jp = (j + 1) & (ny - 1), kpE = (k0 + E) & (nz - 1);
   const size_t P = plane(c);
   const T shift = initial ? (T)0 : pick<T>(prm->mass_shift, prm->f_mass_shift);
   const T sc = initial ? pick<T>(c.inv_h, c.f_inv_h) : pick<T>(c.inv_h / prm->dt, prm->f_sc_div);
-  const int i0 = blockIdx.y * RUN_XCH, i1 = min(i0 + RUN_XCH, nx);
+  const int i0 = blockIdx.y * xch, i1 = min(i0 + xch, nx);
   if (i0 >= i1) return;
   T uw[E];
   ldg_run<T, E>(u + ((size_t)i0 * ny + j) * nz + k0, uw);
@@ -1627,7 +1662,7 @@ __global__ void __launch_bounds__(256, 2)
 k_project_vec(Consts c, const Params* __restrict__ prm, const T* __restrict__ ua,
               const T* __restrict__ va, const T* __restrict__ wa, T* __restrict__ ub,
               T* __restrict__ vb, T* __restrict__ wb, const T* __restrict__ phi, const void* __restrict__ phi_b,
-              T* __restrict__ p, double* __restrict__ partial, int initial) {
+              T* __restrict__ p, double* __restrict__ partial, int initial, int xch) {
   constexpr int E = RunTile<T>::E;
   const T* pb = static_cast<const T*>(phi_b);
   const __nv_bfloat16* pb16 = static_cast<const __nv_bfloat16*>(phi_b);
@@ -1654,7 +1689,7 @@ k_project_vec(Consts c, const Params* __restrict__ prm, const T* __restrict__ ua
   };
   const int nx = c.nx, ny = c.ny, nz = c.nz;
   const int runs = nz / E;
-  const int tj = RunTile<T>::THREADS / runs;
+  const int tj = blockDim.x / runs;
   const int tid = threadIdx.x;
   const int r = tid / runs, k0 = (tid - r * runs) * E;
   const int j = blockIdx.x * tj + r;
@@ -1663,7 +1698,7 @@ k_project_vec(Consts c, const Params* __restrict__ prm, const T* __restrict__ ua
   auto at = [&](int i, int jj, int kk) { return ((size_t)i * ny + jj) * nz + kk; };
   const T gdt = initial ? pick<T>(c.inv_h, c.f_inv_h) : pick<T>(prm->dt * c.inv_h, prm->f_gdt);
   const T hnu = initial ? (T)0 : pick<T>(0.5 * c.nu * prm->dt * c.inv_h * c.inv_h, prm->f_hnu);
-  const int i0 = blockIdx.y * RUN_XCH, i1 = min(i0 + RUN_XCH, nx + 1);
+  const int i0 = blockIdx.y * xch, i1 = min(i0 + xch, nx + 1);
   T smax = 0;
   T phm[E], ph[E], php[E], un[E], un1[E];
 #pragma unroll
@@ -1747,8 +1782,9 @@ k_project_vec(Consts c, const Params* __restrict__ prm, const T* __restrict__ ua
   __syncthreads();
   if (tid == 0) {
     T m = 0;
-    for (int q = 0; q < RunTile<T>::THREADS / 32; ++q) m = fmax(m, wmax[q]);
-    partial[blockIdx.y * gridDim.x + blockIdx.x] = (double)m;
+    for (int q = 0; q < (int)(blockDim.x >> 5); ++q) m = fmax(m, wmax[q]);
+    const int rows = RunTile<T>::THREADS / runs;   // rows of one partial
+    atomic_max_nonneg(&partial[(i0 / PART_PLANES) * (ny / rows) + (blockIdx.x * tj) / rows], (double)m);
   }
 }
 
@@ -1869,6 +1905,34 @@ static size_t rhs_stage_bytes(const Consts& c, int tjr) {
   return (size_t)(3 * (tjr + 2) + (tjr + 1) + 3 * tjr) * c.nz * sizeof(T);
 }
 
+// x planes per block of the streamed explicit stage when the caller gives
+// none: the count that fills whole waves best. A block takes about as long as
+// its planes and one and a half more (first fill, halo planes), all blocks
+// ceil(blocks / slots) times that, with slots the blocks the chip holds. 16
+// planes for every grid left a last wave nearly empty or most SMs idle:
+// 512 x 256 x 256 FP32 0.308 -> 0.297 ms (27 planes, exactly four waves),
+// 384 x 256 x 256 0.259 -> 0.228, 64 x 32 x 32 FP64 0.110 -> 0.019 (2 planes).
+// Blocks of fewer planes read more halo: that costs FP64 little (its pipe
+// bounds the stage), and a small FP32 grid nothing, but larger FP32 grids that
+// share the chip in an ensemble 1.5%, so those keep at least 16 planes.
+template <class T>
+static int rhs_wave_planes(const Consts& c, int yblocks, int per_sm) {
+  const int nx = c.nx;
+  const long long slots = 152ll * (per_sm > 0 ? per_sm : 1);
+  int best = 16;
+  double cost = 1e300;
+  const int least = sizeof(T) == 8 || (long long)nx * c.ny * c.nz <= (1 << 18) ? least_planes(c) : 16;
+  for (int x = least; x <= 40; ++x) {
+    const long long blocks = (long long)yblocks * ((nx + x - 1) / x);
+    const double t = (double)((blocks + slots - 1) / slots) * (x + 1.5);
+    if (t < cost) {
+      cost = t;
+      best = x;
+    }
+  }
+  return best;
+}
+
 template <class T>
 void launch_rhs(const Consts& c, const Fields<T>& f, int cur, cudaStream_t s) {
   {
@@ -1876,7 +1940,12 @@ void launch_rhs(const Consts& c, const Fields<T>& f, int cur, cudaStream_t s) {
     const int threads = RV::TJ * (c.nz / RV::E);
     const size_t sh = (size_t)RV::STAGES * RV::ROWS * c.nz * sizeof(T);
     if (threads % 32 == 0 && threads <= 256 && c.ny % RV::TJ == 0 && sh <= 200 * 1024) {
-      const int XR = c.rhs_planes;
+      int XR = c.rhs_planes;
+      if (!XR) {
+        int per_sm = 0;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_rhs_vec<T>, threads, sh);
+        XR = rhs_wave_planes<T>(c, c.ny / RV::TJ, per_sm);
+      }
       k_rhs_vec<T><<<dim3(c.ny / RV::TJ, (c.nx + XR - 1) / XR), threads, sh, s>>>(
           c, f.prm, f.u[cur], f.v[cur], f.w[cur], f.p, f.n[0], f.n[1], f.n[2], f.d[0], f.d[1],
           f.d[2], XR, inflow_cur_v(c, f), inflow_cur_w(c, f));
@@ -1887,7 +1956,7 @@ void launch_rhs(const Consts& c, const Fields<T>& f, int cur, cudaStream_t s) {
   const size_t stage = rhs_stage_bytes<T>(c, TJR);
   const int rs = (int)std::min<size_t>(std::min(RSTAGES_MAX, c.rhs_stages), (size_t)(210 * 1024) / stage);
   if (rs >= 4 && c.ny % TJR == 0 && (c.nz * sizeof(T)) % 16 == 0) {
-    const int XR = c.rhs_planes;
+    const int XR = c.rhs_planes ? c.rhs_planes : rhs_wave_planes<T>(c, c.ny / TJR, 1);
     k_rhs_pipe<T, TJR><<<dim3(c.ny / TJR, (c.nx + XR - 1) / XR), RTHREADS, rs * stage, s>>>(
         c, f.prm, f.u[cur], f.v[cur], f.w[cur], f.p, f.n[0], f.n[1], f.n[2], f.d[0], f.d[1],
         f.d[2], XR, rs, inflow_cur_v(c, f), inflow_cur_w(c, f));
@@ -2042,9 +2111,9 @@ void launch_mass(const Consts& c, const Fields<T>& f, int cur, cudaStream_t s) {
 
 template <class T>
 void launch_div(const Consts& c, const Fields<T>& f, int cur, bool initial, cudaStream_t s) {
-  if (const int tj = run_rows<T>(c)) {
-    k_div_vec<T><<<dim3(c.ny / tj, (c.nx + RUN_XCH - 1) / RUN_XCH), RunTile<T>::THREADS, 0, s>>>(
-        c, f.prm, f.u[cur], f.v[cur], f.w[cur], f.phi, initial ? 1 : 0);
+  if (const RunShape r = run_shape<T>(c, c.nx, 4); r.rows) {
+    k_div_vec<T><<<dim3(c.ny / r.rows, (c.nx + r.xch - 1) / r.xch), r.threads, 0, s>>>(
+        c, f.prm, f.u[cur], f.v[cur], f.w[cur], f.phi, initial ? 1 : 0, r.xch);
     return;
   }
   k_div<T><<<grid3(c, c.nx), dim3(TK, TJ), 0, s>>>(c, f.prm, f.u[cur], f.v[cur], f.w[cur], f.phi,
@@ -2063,25 +2132,25 @@ template <class T>
 void launch_project_only(const Consts& c, const Fields<T>& f, int cur, bool initial, cudaStream_t s,
                          const T* phi_a, const T* phi_b, const void* phi_b16) {
   if (!phi_a) phi_a = f.phi;
-  if (const int tj = run_rows<T>(c)) {
-    const dim3 grid(c.ny / tj, (c.nx + 1 + RUN_XCH - 1) / RUN_XCH);
+  if (const RunShape r = run_shape<T>(c, c.nx + 1, 8); r.rows) {
+    const dim3 grid(c.ny / r.rows, (c.nx + 1 + r.xch - 1) / r.xch);
     const int ini = initial ? 1 : 0;
     if constexpr (sizeof(T) == 4 && RunTile<T>::E == 4) {
       if (phi_b16) {
-        k_project_vec<T, 2><<<grid, RunTile<T>::THREADS, 0, s>>>(c, f.prm, f.u[cur], f.v[cur], f.w[cur],
+        k_project_vec<T, 2><<<grid, r.threads, 0, s>>>(c, f.prm, f.u[cur], f.v[cur], f.w[cur],
                                                                 f.u[cur ^ 1], f.v[cur ^ 1], f.w[cur ^ 1],
-                                                                phi_a, phi_b16, f.p, f.partial, ini);
+                                                                phi_a, phi_b16, f.p, f.partial, ini, r.xch);
         return;
       }
     }
     if (phi_b)
-      k_project_vec<T, 1><<<grid, RunTile<T>::THREADS, 0, s>>>(c, f.prm, f.u[cur], f.v[cur], f.w[cur],
+      k_project_vec<T, 1><<<grid, r.threads, 0, s>>>(c, f.prm, f.u[cur], f.v[cur], f.w[cur],
                                                               f.u[cur ^ 1], f.v[cur ^ 1], f.w[cur ^ 1],
-                                                              phi_a, phi_b, f.p, f.partial, ini);
+                                                              phi_a, phi_b, f.p, f.partial, ini, r.xch);
     else
-      k_project_vec<T, 0><<<grid, RunTile<T>::THREADS, 0, s>>>(c, f.prm, f.u[cur], f.v[cur], f.w[cur],
+      k_project_vec<T, 0><<<grid, r.threads, 0, s>>>(c, f.prm, f.u[cur], f.v[cur], f.w[cur],
                                                               f.u[cur ^ 1], f.v[cur ^ 1], f.w[cur ^ 1],
-                                                              phi_a, nullptr, f.p, f.partial, ini);
+                                                              phi_a, nullptr, f.p, f.partial, ini, r.xch);
     return;
   }
   k_project<T><<<grid3(c, c.nx + 1), dim3(TK, TJ), 0, s>>>(
@@ -2115,7 +2184,7 @@ void fluid_set_attributes() {
 // blocks of the projection launch (one CFL partial each)
 template <class T>
 int partial_count(const Consts& c) {
-  if (const int tj = run_rows<T>(c)) return c.ny / tj * ((c.nx + 1 + RUN_XCH - 1) / RUN_XCH);
+  if (const int tj = partial_rows<T>(c)) return c.ny / tj * ((c.nx + 1 + PART_PLANES - 1) / PART_PLANES);
   const dim3 g = grid3(c, c.nx + 1);
   return (int)(g.x * g.y * g.z);
 }

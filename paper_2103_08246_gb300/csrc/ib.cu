@@ -599,23 +599,15 @@ template void launch_ib_setup<float>(const Consts&, const Fields<float>&, const 
 // starting at the lowest x cell of the bars; y, z tiles from cell 0 with
 // periodic cells. A marker's cell is floor(X / h) as the kernels compute it
 // (the same FP64 product), so a marker's stencils stay inside its tile's box.
-void ib_bin_bars(const Consts& c, std::vector<double>& Xb, std::vector<int>& tiles, Markers& m) {
+void ib_bin_bars(const Consts& c, std::vector<double>& Xb, std::vector<int>& tiles, Markers& m, std::vector<int>& order) {
   tiles.clear();
+  order.clear();
   m.n_tiles = 0;
   const size_t nb = Xb.size() / 3;
   if (!nb) return;
   m.tx = 8;
   m.ty = c.ny < 16 ? c.ny : 16;
   m.tz = c.nz < 16 ? c.nz : 16;
-  // a plane of few tiles leaves most SMs idle: halve the tiles' transverse
-  // sides down to 4 x 8 while the plane has fewer than 32 (64 x 32 x 32 FP64:
-  // 3.78 -> 3.22 ms per 10 steps; going on to one tile per SM slows ensembles,
-  // which fill the SMs with members, by 4%)
-  while ((m.ty > 4 || m.tz > 8) && (c.ny / m.ty) * (c.nz / m.tz) < 32) {
-    if (m.ty > 4 && m.ty >= m.tz) m.ty /= 2;
-    else if (m.tz > 8) m.tz /= 2;
-    else m.ty /= 2;
-  }
   auto cell = [&](double x, int n, bool periodic) {
     long long q = (long long)std::floor(x * c.inv_h);
     if (periodic) q = ((q % n) + n) % n;
@@ -627,29 +619,53 @@ void ib_bin_bars(const Consts& c, std::vector<double>& Xb, std::vector<int>& til
     x0 = std::min(x0, cx);
     x1 = std::max(x1, cx);
   }
-  const int ntx = (x1 - x0) / m.tx + 1;
+  // stable sort of the markers by tile; the first marker of every tile in `count`
+  std::vector<int> count;
+  auto sort_by_tile = [&](std::vector<int>& pos) {
+    const int ntx = (x1 - x0) / m.tx + 1, nty = (c.ny + m.ty - 1) / m.ty, ntz = (c.nz + m.tz - 1) / m.tz;
+    count.assign((size_t)ntx * nty * ntz + 1, 0);
+    std::vector<int> key(nb);
+    for (size_t b = 0; b < nb; ++b) {
+      const int tx = (cell(Xb[3 * b], c.nx, false) - x0) / m.tx;
+      const int ty = cell(Xb[3 * b + 1], c.ny, true) / m.ty;
+      const int tz = cell(Xb[3 * b + 2], c.nz, true) / m.tz;
+      key[b] = (tx * nty + ty) * ntz + tz;
+      ++count[key[b] + 1];
+    }
+    for (size_t t = 0; t + 1 < count.size(); ++t) count[t + 1] += count[t];
+    std::vector<int> at(count.begin(), count.end() - 1);
+    pos.resize(nb);
+    std::vector<double> sorted(Xb.size());
+    for (size_t b = 0; b < nb; ++b) {
+      pos[b] = at[key[b]]++;
+      for (int q = 0; q < 3; ++q) sorted[3 * (size_t)pos[b] + q] = Xb[3 * b + q];
+    }
+    Xb.swap(sorted);
+  };
+  std::vector<int> pos;
+  sort_by_tile(pos);
+  // a plane of few tiles leaves most SMs idle: halve the tiles' transverse
+  // sides down to 4 x 8 while the plane has fewer than 32 (64 x 32 x 32 FP64:
+  // 3.78 -> 3.22 ms per 10 steps; going on to one tile per SM slows ensembles,
+  // which fill the SMs with members, by 4%). The markers are then sorted once
+  // more, and `order` gives each marker's place in the 16 x 16 order, in which
+  // they are reported whatever the tiles.
+  const int ty = m.ty, tz = m.tz;
+  while ((m.ty > 4 || m.tz > 8) && (c.ny / m.ty) * (c.nz / m.tz) < 32) {
+    if (m.ty > 4 && m.ty >= m.tz) m.ty /= 2;
+    else if (m.tz > 8) m.tz /= 2;
+    else m.ty /= 2;
+  }
+  if (m.ty != ty || m.tz != tz) {
+    sort_by_tile(pos);
+    order.resize(nb);
+    for (size_t b = 0; b < nb; ++b) order[pos[b]] = (int)b;
+  }
   const int nty = (c.ny + m.ty - 1) / m.ty, ntz = (c.nz + m.tz - 1) / m.tz;
-  const size_t ntile = (size_t)ntx * nty * ntz;
-  std::vector<int> key(nb), count(ntile + 1, 0);
-  for (size_t b = 0; b < nb; ++b) {
-    const int tx = (cell(Xb[3 * b], c.nx, false) - x0) / m.tx;
-    const int ty = cell(Xb[3 * b + 1], c.ny, true) / m.ty;
-    const int tz = cell(Xb[3 * b + 2], c.nz, true) / m.tz;
-    key[b] = (tx * nty + ty) * ntz + tz;
-    ++count[key[b] + 1];
-  }
-  for (size_t t = 0; t < ntile; ++t) count[t + 1] += count[t];
-  std::vector<double> sorted(Xb.size());
-  std::vector<int> pos(count.begin(), count.end() - 1);
-  for (size_t b = 0; b < nb; ++b) {
-    const int d = pos[key[b]]++;
-    for (int q = 0; q < 3; ++q) sorted[3 * (size_t)d + q] = Xb[3 * b + q];
-  }
-  Xb.swap(sorted);
-  for (size_t t = 0; t < ntile; ++t) {
+  for (size_t t = 0; t + 1 < count.size(); ++t) {
     if (count[t + 1] == count[t]) continue;
-    const int tz = (int)(t % ntz), ty = (int)((t / ntz) % nty), tx = (int)(t / ((size_t)ntz * nty));
-    tiles.insert(tiles.end(), {x0 + tx * m.tx, ty * m.ty, tz * m.tz, count[t], count[t + 1]});
+    const int iz = (int)(t % ntz), iy = (int)((t / ntz) % nty), ix = (int)(t / ((size_t)ntz * nty));
+    tiles.insert(tiles.end(), {x0 + ix * m.tx, iy * m.ty, iz * m.tz, count[t], count[t + 1]});
   }
   m.n_tiles = (int)(tiles.size() / 5);
 }

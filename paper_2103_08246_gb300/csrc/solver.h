@@ -201,8 +201,9 @@ template <class T> void launch_ib(const Consts& c, const Fields<T>& f, const Mar
 void ib_set_attributes();
 template <class T> void launch_ib_setup(const Consts& c, const Fields<T>& f, const Markers& m, cudaStream_t s);
 // bin the bar markers (3 doubles each, sorted in place) into tiles; fills
-// the tile table (5 ints per tile) and the tile shape of m
-void ib_bin_bars(const Consts& c, std::vector<double>& Xb, std::vector<int>& tiles, Markers& m);
+// the tile table (5 ints per tile) and the tile shape of m; order: where small
+// planes take smaller tiles, each marker's place in the reported order
+void ib_bin_bars(const Consts& c, std::vector<double>& Xb, std::vector<int>& tiles, Markers& m, std::vector<int>& order);
 
 // ---- slab.cu
 void slab_tables(const Consts& c, const SlabDev& sd, cudaStream_t s);
