@@ -83,9 +83,10 @@ extern "C" {
                                    the step runs AF_Y and AF_Z and this stage
                                    launches nothing)                          */
 #define IBM_STAGE_DHT_2D    14  /* both transforms of every x plane in one pass
-                                   (used by the pressure solve when ny = nz =
-                                   256; otherwise the solve runs DHT_Y and
-                                   DHT_Z and this stage launches nothing)     */
+                                   (IBM_FP32 and IBM_MIXED, when ny = nz = 256
+                                   or ny nz <= 32,768 with both at most 256;
+                                   otherwise the solve runs DHT_Y and DHT_Z and
+                                   this stage launches nothing)               */
 #define IBM_STAGE_TC_PASS   15  /* one tensor-core transform pass (X H)^T over every
                                    x plane (IBM_MIXED with square planes of 32,
                                    64, 128 or 256; otherwise nothing), split
@@ -182,13 +183,14 @@ typedef struct {
    * cell's solid fraction (zero inside the solid); the bars then carry no
    * markers. [0] */
   int bar_forcing;
-  /* IBM_MIXED with 256 x 256 transverse planes. 0: the refinement's
-   * predictor is the FP32 FFT solve and the correction's transforms run on
-   * the tensor cores with the single TF32 product. 1: both solves on the
-   * tensor cores, the predictor with the single and the correction with the
-   * split TF32 products. Both leave the FP32 rounding of the stored result
-   * as the error (the final error is the product of the two solves' relative
-   * errors); 0 is faster. Other plane sizes always take 1's scheme. [0] */
+  /* IBM_MIXED. 0: at 256 x 256 transverse planes the refinement's predictor is
+   * the FP32 FFT solve and the correction's transforms run on the tensor cores
+   * in bfloat16; at smaller planes (IBM_STAGE_DHT_2D) both solves are the FP32
+   * FFT. 1: both solves on the tensor cores, the predictor with the single (at
+   * 256 x 256) and the correction with the split TF32 products. Both leave the
+   * FP32 rounding of the stored result as the error (the final error is the
+   * product of the two solves' relative errors); 0 is faster. Planes without a
+   * one-pass FFT always take 1's scheme. [0] */
   int mixed_tc_predictor;
 } ibm_options;
 

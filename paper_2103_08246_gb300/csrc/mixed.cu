@@ -326,8 +326,9 @@ static void transform2d(const Consts& c, const Hartley& H, const float* in, floa
 // residual rounded to bfloat16, the tensor-core transforms on bfloat16
 // operands with FP32 accumulation, the Thomas sweeps in FP32 arithmetic on
 // bfloat16 storage (relative error about 2^-8 altogether), half the bytes of
-// an FP32 correction. Otherwise both solves run on the tensor cores with FP32
-// storage, the predictor with the single TF32 product where it exists (256),
+// an FP32 correction. Planes that fit one SM's shared memory take the FP32 FFT
+// for both solves. Otherwise (and with mixed_tc_predictor) both solves run on
+// the tensor cores with FP32 storage, the predictor with the single TF32 product where it exists (256),
 // the correction with the split products. Scratch: e[0], e[1], e[2]
 // (bfloat16 correction: the first halves of e[0] and e[2]).
 void launch_poisson_mixed(const Consts& c, const Fields<float>& f, const float* Hy, const float* Hz,
@@ -353,6 +354,20 @@ void launch_poisson_mixed(const Consts& c, const Fields<float>& f, const float* 
     launch_poisson_x_bf16(c, f, r16, s);
     tc_rows_times_h_bf16(r16, H16_img, w16, c.nx, err, s, c.sm_reserved);
     tc_rows_times_h_bf16(w16, H16_img, r16, c.nx, err, s, c.sm_reserved);
+    return;
+  }
+  if (!c.mixed_tc && dht2d_plane_supported(c.ny, c.nz)) {
+    // planes that fit one SM: both solves by the FP32 FFT (relative error near
+    // FP32 rounding each). Four tensor-core passes per solve write and read the
+    // field through L2 and hold every SM with one persistent CTA: 256 planes of
+    // 128 x 128 0.206 ms, 0.135 here
+    launch_dht2d_on(c, f, D, x0, s);
+    launch_poisson_x_on(c, f, x0, s);
+    launch_dht2d_on(c, f, x0, x0, s);
+    launch_residual(c, D, x0, t1, s);
+    launch_dht2d_on(c, f, t1, t1, s);
+    launch_poisson_x_on(c, f, t1, s);
+    launch_dht2d_on(c, f, t1, t1, s);
     return;
   }
   // predictor: x0 = L^-1 D

@@ -27,6 +27,7 @@
 
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cmath>
 #include <type_traits>
 
@@ -112,18 +113,7 @@ k_dht(T* __restrict__ data, int n, int logn, int W, int lines_per_group, size_t 
   }
 }
 
-// ---- 256-point transforms of one warp (n = 256)
-// Four-step FFT, N = 8 x 32 with n = l + 32 m, k = p + 8 q: lane l holds
-// z[l + 32 m], m = 0..7; an 8-point DFT over m in registers and the twiddles
-// W_256^{l p} leave, for every p, a 32-point DFT over the lanes l. Those are
-// split again as 32 = 8 x 4 (l = a + 4 b, q = e + 8 f): a transpose through
-// the warp's shared buffer gives lane 4 p + a the values b = 0..7, an
-// in-register 8-point DFT over b, twiddles W_32^{a e}, and a 4-point DFT
-// across the lane quad (two shuffle stages, factors +-1 and -i only); lane
-// 4 p + a then holds Z[p + 8 e + 64 f] in register e, f = brev2(a). Two real
-// lines a, b travel as z = a + i b; the Hartley outputs need Z_k and Z_{N-k},
-// which every lane reads back from the shared buffer for k = l + 32 t, so
-// the outputs come out in the input's distribution (lane l: l + 32 t).
+// ---- transforms in registers
 template <class T>
 struct Cx {
   T r, i;
@@ -175,237 +165,12 @@ __device__ inline void dft8(Cx<T> (&x)[8]) {
 }
 
 template <class T>
-__device__ inline T shfl(T v, int lane) { return __shfl_sync(0xffffffffu, v, lane); }
-template <class T>
-__device__ inline T shfl_x(T v, int m) { return __shfl_xor_sync(0xffffffffu, v, m); }
-
-// Twiddles a lane needs in every transform, read once from the shared table
-// tw (W_256^t = (cos, -sin)(2 pi t / 256), t = 0..255): W^{l p} after the
-// 8-point DFTs, and per cross-lane stage (distance d) a sign and a factor
-// that turn both halves of the butterfly into one expression,
-//   lower lane: x + o = (o + x) * 1,   upper lane: (o - x) * W.
-// Twiddles W^{l p} of the first pass, read once from the shared table tw
-// (W_256^t = (cos, -sin)(2 pi t / 256), t = 0..255).
-template <class T>
-struct LaneTw {
-  Cx<T> tp[8];
-};
-
-template <class T>
-__device__ inline LaneTw<T> lane_twiddles(const Cx<T>* tw) {
-  LaneTw<T> lt;
-  const int l = threadIdx.x & 31;
-#pragma unroll
-  for (int p = 0; p < 8; ++p) lt.tp[p] = tw[(l * p) & 255];
-  return lt;
-}
-
-// per-warp shared scratch: the transpose [8][36] and then Z at k + 4 (k / 64)
-constexpr int WFFT_BUF = 8 * 36;
-__device__ inline int zslot(int k) { return k + 4 * (k >> 6); }
-
-template <class T>
-__device__ inline void warp_hartley256(Cx<T> (&x)[8], const LaneTw<T>& lt, const Cx<T>* tw,
-                                       Cx<T>* wb, T (&ha)[8], T (&hb)[8]) {
-  const int l = threadIdx.x & 31;
-  dft8(x);
-#pragma unroll
-  for (int p = 1; p < 8; ++p) x[p] = cmul(x[p], lt.tp[p]);
-  // transpose: lane 4 pp + a takes Y_{a + 4 b}[pp], b = 0..7
-#pragma unroll
-  for (int p = 0; p < 8; ++p) wb[p * 36 + l] = x[p];
-  __syncwarp();
-  const int pp = l >> 2, a = l & 3;
-#pragma unroll
-  for (int b = 0; b < 8; ++b) x[b] = wb[pp * 36 + a + 4 * b];
-  dft8(x);
-#pragma unroll
-  for (int e = 1; e < 8; ++e) x[e] = cmul(x[e], tw[(8 * a * e) & 255]);   // W_32^{a e}
-  // 4-point DFT across the quad, decimation in frequency
-  {
-    const bool up = (a & 2) != 0, rot = (a & 3) == 3;
-    const T sg = up ? (T)-1 : (T)1;
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const Cx<T> o = {shfl_x(x[e].r, 2), shfl_x(x[e].i, 2)};
-      const Cx<T> t = {o.r + sg * x[e].r, o.i + sg * x[e].i};
-      x[e] = rot ? Cx<T>{t.i, -t.r} : t;   // W_4^1 = -i on the odd upper lane
-    }
-  }
-  {
-    const T sg = (a & 1) ? (T)-1 : (T)1;
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const Cx<T> o = {shfl_x(x[e].r, 1), shfl_x(x[e].i, 1)};
-      x[e] = {o.r + sg * x[e].r, o.i + sg * x[e].i};
-    }
-  }
-  __syncwarp();   // the transpose has been read by every lane
-  const int f = ((a & 1) << 1) | (a >> 1);
-#pragma unroll
-  for (int e = 0; e < 8; ++e) wb[zslot(pp + 8 * e + 64 * f)] = x[e];
-  __syncwarp();
-#pragma unroll
-  for (int t = 0; t < 8; ++t) {
-    const int k = l + 32 * t;
-    const Cx<T> zk = wb[zslot(k)], zr = wb[zslot((256 - k) & 255)];
-    ha[t] = (T)0.5 * (zk.r - zk.i + zr.r + zr.i);
-    hb[t] = (T)0.5 * (zk.r + zk.i - zr.r + zr.i);
-  }
-  __syncwarp();   // the buffer is free for the warp's next transform
-}
-
-template <class T>
 __device__ inline void load_twiddles(Cx<T>* tw, const T* g) {
   for (int t = threadIdx.x; t < 128; t += blockDim.x) {
     tw[t] = {g[2 * t], g[2 * t + 1]};
     tw[t + 128] = {-g[2 * t], -g[2 * t + 1]};   // W^{t+128} = -W^t
   }
   __syncthreads();
-}
-
-// z lines (contiguous rows of 256): one warp per pair of rows, in place
-template <class T>
-__global__ void __launch_bounds__(256) k_dht_z256(T* __restrict__ data, int nrows, const T* __restrict__ twg) {
-  __shared__ Cx<T> tw[256];
-  __shared__ Cx<T> wbuf[8][WFFT_BUF];
-  load_twiddles(tw, twg);
-  const LaneTw<T> lt = lane_twiddles(tw);
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int l = threadIdx.x & 31;
-  if (2 * warp + 1 >= nrows + 1) return;
-  T* a = data + (size_t)(2 * warp) * 256;
-  T* b = a + 256;
-  Cx<T> x[8];
-#pragma unroll
-  for (int m = 0; m < 8; ++m) x[m] = {a[l + 32 * m], b[l + 32 * m]};
-  T ha[8], hb[8];
-  warp_hartley256(x, lt, tw, wbuf[threadIdx.x >> 5], ha, hb);
-  // lane l holds outputs l + 32 t: coalesced rows
-#pragma unroll
-  for (int t = 0; t < 8; ++t) {
-    a[l + 32 * t] = ha[t];
-    b[l + 32 * t] = hb[t];
-  }
-}
-
-// y lines (columns of a plane, ny = 256): a block stages a 256 x 32 tile
-// (coalesced rows), 16 warps transform two columns each, the tile is stored back.
-// Tile element (r, c) sits at r * 33 + ((c + (r >> 5)) & 31): the row pad
-// spreads the column reads and writes (rows l + 32 t across the lanes) over
-// the banks. Each warp's FFT scratch follows the tile in shared memory.
-__device__ inline int ytile(int r, int c) { return r * 33 + ((c + (r >> 5)) & 31); }
-
-template <class T>
-__global__ void __launch_bounds__(512) k_dht_y256(T* __restrict__ data, int nz, const T* __restrict__ twg) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ Cx<T> tw[256];
-  T* s = reinterpret_cast<T*>(smem_raw);   // [256][33]
-  Cx<T>* wbuf = reinterpret_cast<Cx<T>*>(s + 256 * 33) + (threadIdx.x >> 5) * WFFT_BUF;
-  const int ct = nz / 32;
-  const int plane = blockIdx.x / ct, c0 = (blockIdx.x - plane * ct) * 32;
-  T* base = data + (size_t)plane * 256 * nz + c0;
-  for (int e = threadIdx.x; e < 256 * 32; e += blockDim.x) {
-    const int r = e >> 5, c = e & 31;
-    s[ytile(r, c)] = base[(size_t)r * nz + c];
-  }
-  load_twiddles(tw, twg);   // includes __syncthreads
-  const LaneTw<T> lt = lane_twiddles(tw);
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  Cx<T> x[8];
-#pragma unroll
-  for (int m = 0; m < 8; ++m) x[m] = {s[ytile(l + 32 * m, 2 * w)], s[ytile(l + 32 * m, 2 * w + 1)]};
-  T ha[8], hb[8];
-  warp_hartley256(x, lt, tw, wbuf, ha, hb);
-  __syncthreads();
-#pragma unroll
-  for (int t = 0; t < 8; ++t) {
-    s[ytile(l + 32 * t, 2 * w)] = ha[t];
-    s[ytile(l + 32 * t, 2 * w + 1)] = hb[t];
-  }
-  __syncthreads();
-  for (int e = threadIdx.x; e < 256 * 32; e += blockDim.x) {
-    const int r = e >> 5, c = e & 31;
-    base[(size_t)r * nz + c] = s[ytile(r, c)];
-  }
-}
-
-// Both transforms of one 256 x 256 x-plane in a single pass: a cluster of 8
-// CTAs holds the plane as eight 256 x 32 column tiles (CTA q: columns
-// 32 q .. 32 q + 31). Each CTA transforms its 32 columns along y (two per
-// warp per round), the cluster synchronises, then CTA q transforms rows
-// 32 q .. 32 q + 31 along z (two per warp per round), gathering each row's
-// eight 32-value pieces from the eight tiles through distributed shared
-// memory and storing the finished rows straight to global memory. A last
-// cluster barrier keeps every tile alive until all its readers are done.
-// The plane is read and written once.
-constexpr int DHT2D_CLUSTER = 8;
-constexpr int DHT2D_THREADS = 256;
-template <class T>
-__global__ void __cluster_dims__(DHT2D_CLUSTER, 1, 1) __launch_bounds__(DHT2D_THREADS, sizeof(T) == 4 ? 4 : 2)
-k_dht2d_256(T* __restrict__ data, const T* __restrict__ twy) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ Cx<T> tw[256];
-  T* s = reinterpret_cast<T*>(smem_raw);   // [256][33], element (r, c) at ytile(r, c)
-  Cx<T>* wbuf = reinterpret_cast<Cx<T>*>(s + 256 * 33) + (threadIdx.x >> 5) * WFFT_BUF;
-  cg::cluster_group cl = cg::this_cluster();
-  const int q = (int)cl.block_rank();
-  const int plane = blockIdx.x / DHT2D_CLUSTER;
-  T* pbase = data + (size_t)plane * 256 * 256;
-  {
-    const T* base = pbase + 32 * q;
-    constexpr int PER = 256 * 32 / DHT2D_THREADS;   // 32 values per thread
-    T buf[PER];
-#pragma unroll
-    for (int t = 0; t < PER; ++t) {
-      const int e = threadIdx.x + t * DHT2D_THREADS;
-      buf[t] = base[(size_t)(e >> 5) * 256 + (e & 31)];
-    }
-#pragma unroll
-    for (int t = 0; t < PER; ++t) {
-      const int e = threadIdx.x + t * DHT2D_THREADS;
-      s[ytile(e >> 5, e & 31)] = buf[t];
-    }
-  }
-  load_twiddles(tw, twy);   // includes __syncthreads
-  const LaneTw<T> lt = lane_twiddles(tw);
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  constexpr int NW = DHT2D_THREADS / 32;
-  // y: column pairs (2 cp, 2 cp + 1) of this tile
-  for (int cp = w; cp < 16; cp += NW) {
-    Cx<T> x[8];
-#pragma unroll
-    for (int m = 0; m < 8; ++m) x[m] = {s[ytile(l + 32 * m, 2 * cp)], s[ytile(l + 32 * m, 2 * cp + 1)]};
-    T ha[8], hb[8];
-    warp_hartley256(x, lt, tw, wbuf, ha, hb);
-#pragma unroll
-    for (int t = 0; t < 8; ++t) {
-      s[ytile(l + 32 * t, 2 * cp)] = ha[t];
-      s[ytile(l + 32 * t, 2 * cp + 1)] = hb[t];
-    }
-  }
-  cl.sync();   // every tile transformed along y (ny = nz: the same twiddles serve z)
-  // z: row pairs of this CTA; value (r, k) lives in tile k / 32 at column k % 32
-  for (int rp = w; rp < 16; rp += NW) {
-    const int r0 = 32 * q + 2 * rp;
-    Cx<T> x[8];
-#pragma unroll
-    for (int m = 0; m < 8; ++m) {
-      const T* t = cl.map_shared_rank(s, m);
-      x[m] = {t[ytile(r0, l)], t[ytile(r0 + 1, l)]};
-    }
-    T ha[8], hb[8];
-    warp_hartley256(x, lt, tw, wbuf, ha, hb);
-    // lane l holds outputs l + 32 t of both rows: coalesced rows
-    T* a = pbase + (size_t)r0 * 256;
-    T* b = a + 256;
-#pragma unroll
-    for (int t = 0; t < 8; ++t) {
-      a[l + 32 * t] = ha[t];
-      b[l + 32 * t] = hb[t];
-    }
-  }
-  cl.sync();   // no tile is released while another CTA may still read it
 }
 
 // ---- FP32: both transforms of a 256 x 256 plane with thread-level radix-16
@@ -440,9 +205,10 @@ constexpr int R16_THREADS = 512;
 constexpr int R16_ROW = 257;   // complex stride of the separation buffer [32][257]
 constexpr size_t R16_SMEM = (size_t)32 * R16_ROW * sizeof(Cx<float>);   // >= the transpose's 16 x 16 x 32
 
-__device__ __forceinline__ void dft4_cx(Cx<float>& a0, Cx<float>& a1, Cx<float>& a2, Cx<float>& a3) {
-  const Cx<float> t0 = {a0.r + a2.r, a0.i + a2.i}, t1 = {a0.r - a2.r, a0.i - a2.i};
-  const Cx<float> t2 = {a1.r + a3.r, a1.i + a3.i}, t3 = {a1.r - a3.r, a1.i - a3.i};
+template <class T>
+__device__ __forceinline__ void dft4_cx(Cx<T>& a0, Cx<T>& a1, Cx<T>& a2, Cx<T>& a3) {
+  const Cx<T> t0 = {a0.r + a2.r, a0.i + a2.i}, t1 = {a0.r - a2.r, a0.i - a2.i};
+  const Cx<T> t2 = {a1.r + a3.r, a1.i + a3.i}, t3 = {a1.r - a3.r, a1.i - a3.i};
   a0 = {t0.r + t2.r, t0.i + t2.i};
   a2 = {t0.r - t2.r, t0.i - t2.i};
   a1 = {t1.r + t3.i, t1.i - t3.r};   // t1 - i t3
@@ -450,8 +216,9 @@ __device__ __forceinline__ void dft4_cx(Cx<float>& a0, Cx<float>& a1, Cx<float>&
 }
 
 // (a + i b) W16^e for the exponents e = n2 k1 of the 4 x 4 split
-__device__ __forceinline__ Cx<float> w16(Cx<float> a, int e) {
-  const float C = 0.92387953251128675613f, S = 0.38268343236508977173f, R = 0.70710678118654752440f;
+template <class T>
+__device__ __forceinline__ Cx<T> w16(Cx<T> a, int e) {
+  const T C = (T)0.92387953251128675613, S = (T)0.38268343236508977173, R = (T)0.70710678118654752440;
   switch (e) {
     case 1: return {a.r * C + a.i * S, a.i * C - a.r * S};
     case 2: return {(a.r + a.i) * R, (a.i - a.r) * R};
@@ -466,7 +233,8 @@ __device__ __forceinline__ Cx<float> w16(Cx<float> a, int e) {
 // in-register 16-point DFT, natural order in and out: n = 4 n1 + n2,
 // k = k1 + 4 k2, a 4-point DFT over n1, twiddles W16^{n2 k1}, a 4-point DFT
 // over n2
-__device__ __forceinline__ void dft16(Cx<float> (&x)[16]) {
+template <class T>
+__device__ __forceinline__ void dft16(Cx<T> (&x)[16]) {
 #pragma unroll
   for (int n2 = 0; n2 < 4; ++n2) dft4_cx(x[n2], x[4 + n2], x[8 + n2], x[12 + n2]);
 #pragma unroll
@@ -480,7 +248,7 @@ __device__ __forceinline__ void dft16(Cx<float> (&x)[16]) {
   for (int a = 0; a < 4; ++a)
 #pragma unroll
     for (int b = a + 1; b < 4; ++b) {
-      const Cx<float> t = x[4 * a + b];
+      const Cx<T> t = x[4 * a + b];
       x[4 * a + b] = x[4 * b + a];
       x[4 * b + a] = t;
     }
@@ -501,8 +269,8 @@ __device__ __forceinline__ void cluster_wait_acquire() {
 // transpose, and the outer DFT: on return x[k2] = Z(k1 + 16 k2) of the lane's
 // line pair, k1 = the warp index. `pre_wait` runs between the transpose's
 // stores and loads (the cluster arrive of phase y).
-template <class F>
-__device__ __forceinline__ void r16_fft(Cx<float> (&x)[16], const Cx<float>* tw, Cx<float>* buf, int w, int l,
+template <class T, class F>
+__device__ __forceinline__ void r16_fft(Cx<T> (&x)[16], const Cx<T>* tw, Cx<T>* buf, int w, int l,
                                         F pre_wait) {
   dft16(x);
 #pragma unroll
@@ -513,6 +281,23 @@ __device__ __forceinline__ void r16_fft(Cx<float> (&x)[16], const Cx<float>* tw,
   for (int j0 = 0; j0 < 16; ++j0) x[j0] = buf[(w * 16 + j0) * 32 + l];
   dft16(x);
   __syncthreads();   // the transpose buffer is free for the separation buffer
+}
+
+// the mirrored pair of a separation: Z_k and Z_{N-k} give the Hartley values
+// k and N - k of both packed lines (times two) from four sums
+template <class T>
+struct Sep {
+  T ak, bk, am, bm;   // lines a, b at k, then at N - k
+};
+template <class T>
+__device__ __forceinline__ Sep<T> separate(Cx<T> zk, Cx<T> zm) {
+  const T sr = zk.r + zm.r, dr = zk.r - zm.r, si = zk.i + zm.i, di = zk.i - zm.i;
+  return {sr - di, si + dr, sr + di, si - dr};
+}
+// k = 0 and N / 2 are their own mirrors; z0, zh their values: a, b at 0, then at N / 2
+template <class T>
+__device__ __forceinline__ Sep<T> separate_ends(Cx<T> z0, Cx<T> zh) {
+  return {z0.r + z0.r, z0.i + z0.i, zh.r + zh.r, zh.i + zh.i};
 }
 
 __global__ void __cluster_dims__(R16_CLUSTER, 1, 1) __launch_bounds__(R16_THREADS, 2)
@@ -553,11 +338,11 @@ k_dht2d_r16(const float* in, float* out, const float* __restrict__ twy) {
       const int k = l + 32 * v;
       const int kr = k == 0 ? 128 : 256 - k;   // k = 0 and 128 are their own mirrors
       const Cx<float> zk = Zp[k], zr = Zp[kr];
-      const Cx<float> mk = k == 0 ? zk : zr, mr = k == 0 ? zr : zk;
-      P[r16_perm(k, za)] = 0.5f * (zk.r - zk.i + mk.r + mk.i);
-      P[r16_perm(k, zb)] = 0.5f * (zk.r + zk.i - mk.r + mk.i);
-      P[r16_perm(kr, za)] = 0.5f * (zr.r - zr.i + mr.r + mr.i);
-      P[r16_perm(kr, zb)] = 0.5f * (zr.r + zr.i - mr.r + mr.i);
+      const Sep<float> o = k == 0 ? separate_ends(zk, zr) : separate(zk, zr);
+      P[r16_perm(k, za)] = o.ak;
+      P[r16_perm(k, zb)] = o.bk;
+      P[r16_perm(kr, za)] = o.am;
+      P[r16_perm(kr, zb)] = o.bm;
     }
   }
   cluster_arrive_release();
@@ -583,13 +368,309 @@ k_dht2d_r16(const float* in, float* out, const float* __restrict__ twy) {
       const int k = l + 32 * v;
       const int kr = k == 0 ? 128 : 256 - k;
       const Cx<float> zk = Zp[k], zr = Zp[kr];
-      const Cx<float> mk = k == 0 ? zk : zr, mr = k == 0 ? zr : zk;
-      ra[k] = 0.5f * (zk.r - zk.i + mk.r + mk.i);
-      rb[k] = 0.5f * (zk.r + zk.i - mk.r + mk.i);
-      ra[kr] = 0.5f * (zr.r - zr.i + mr.r + mr.i);
-      rb[kr] = 0.5f * (zr.r + zr.i - mr.r + mr.i);
+      const Sep<float> o = k == 0 ? separate_ends(zk, zr) : separate(zk, zr);
+      ra[k] = 0.25f * o.ak;   // a half for each direction's separation
+      rb[k] = 0.25f * o.bk;
+      ra[kr] = 0.25f * o.am;
+      rb[kr] = 0.25f * o.bm;
     }
   }
+}
+
+
+// ---- one direction, lines of 4 to 256 points (FP64 always; FP32 beyond the planes below)
+// A CTA transforms 2 P real lines as P complex ones, N = R1 R2 with radices up
+// to 16: R1-point DFTs of the elements j0 + R2 m in registers, twiddles
+// W^{j0 k1}, R2-point DFTs over j0 after one trip through shared memory, and
+// the separation on the way back to global memory. Two barriers where the
+// radix-2 form (k_dht) has log2 N + 1. In FP64 the transforms are bound by the
+// FP64 pipe (two instructions per clock and SM): about 12 instructions per
+// value and direction plus two for the separation, against 18 to 24 of k_dht
+// and of the warp-level 256-point form that was here; the blocks are small, so
+// several share an SM and all SMs get the same number. FP64, y + z: 512 planes of
+// 256 x 256 2.26 -> 1.88 ms, 256 of 128 x 128 0.344 -> 0.230.
+template <class T, int R>
+__device__ __forceinline__ void dft_r(Cx<T> (&x)[R]) {
+  if constexpr (R == 16) dft16(x);
+  else if constexpr (R == 8) dft8(x);
+  else if constexpr (R == 4) dft4_cx(x[0], x[1], x[2], x[3]);
+}
+constexpr int DHT1_PAIRS = 16;
+// y: columns of a plane (positions nz apart); pairs (c, c + P) of a tile of 2 P columns
+template <class T, int R1, int R2>
+__global__ void __launch_bounds__(256, 2) k_dht1_y(T* __restrict__ data, int nz, int P, const T* __restrict__ twg) {
+  constexpr int N = R1 * R2;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  Cx<T>* S = reinterpret_cast<Cx<T>*>(smem_raw);   // [N][P], wavenumber k1 + R1 k2 at row k1 R2 + k2
+  Cx<T>* tw = S + N * P;
+  const int tiles = nz / (2 * P), lp = 31 - __clz(P);
+  const int pl = blockIdx.x / tiles;
+  T* base = data + (size_t)pl * N * nz + (size_t)(blockIdx.x - pl * tiles) * 2 * P;
+  for (int q = threadIdx.x; q < N / 2; q += blockDim.x) {
+    tw[q] = {twg[2 * q], twg[2 * q + 1]};
+    tw[q + N / 2] = {-twg[2 * q], -twg[2 * q + 1]};
+  }
+  __syncthreads();
+  for (int q = threadIdx.x; q < P * R2; q += blockDim.x) {
+    const int c = q & (P - 1), j0 = q >> lp;
+    const T* col = base + (size_t)j0 * nz + c;
+    Cx<T> x[R1];
+#pragma unroll
+    for (int m = 0; m < R1; ++m) x[m] = {col[(size_t)(m * R2) * nz], col[(size_t)(m * R2) * nz + P]};
+    dft_r<T, R1>(x);
+#pragma unroll
+    for (int k1 = 0; k1 < R1; ++k1) S[(j0 + R2 * k1) * P + c] = k1 && j0 ? cmul(x[k1], tw[j0 * k1]) : x[k1];
+  }
+  __syncthreads();
+  if constexpr (R2 > 1) {
+    for (int q = threadIdx.x; q < P * R1; q += blockDim.x) {
+      Cx<T>* s = S + (q >> lp) * R2 * P + (q & (P - 1));
+      Cx<T> x[R2];
+#pragma unroll
+      for (int j = 0; j < R2; ++j) x[j] = s[j * P];
+      dft_r<T, R2>(x);
+#pragma unroll
+      for (int j = 0; j < R2; ++j) s[j * P] = x[j];
+    }
+    __syncthreads();
+  }
+  for (int q = threadIdx.x; q < P * (N / 2); q += blockDim.x) {
+    const int c = q & (P - 1), k = q >> lp, km = k ? N - k : N / 2;
+    const Cx<T> zk = S[((k % R1) * R2 + k / R1) * P + c], zm = S[((km % R1) * R2 + km / R1) * P + c];
+    const Sep<T> o = k ? separate(zk, zm) : separate_ends(zk, zm);
+    T* a = base + (size_t)k * nz + c;
+    T* b = base + (size_t)km * nz + c;
+    a[0] = (T)0.5 * o.ak;
+    a[P] = (T)0.5 * o.bk;
+    b[0] = (T)0.5 * o.am;
+    b[P] = (T)0.5 * o.bm;
+  }
+}
+// z: contiguous lines; pairs (r, r + P) of 2 P consecutive rows
+template <class T, int R1, int R2>
+__global__ void __launch_bounds__(256, 2) k_dht1_z(T* __restrict__ data, int P, const T* __restrict__ twg) {
+  constexpr int N = R1 * R2;
+  constexpr int LD = N + (R2 > 1 ? R1 : 1);   // one slot of padding per R2
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  Cx<T>* S = reinterpret_cast<Cx<T>*>(smem_raw);   // [P][LD], position p at p + p / R2
+  Cx<T>* tw = S + LD * P;
+  T* base = data + (size_t)blockIdx.x * 2 * P * N;
+  auto at = [](int p) { return R2 > 1 ? p + p / R2 : p; };
+  for (int q = threadIdx.x; q < N / 2; q += blockDim.x) {
+    tw[q] = {twg[2 * q], twg[2 * q + 1]};
+    tw[q + N / 2] = {-twg[2 * q], -twg[2 * q + 1]};
+  }
+  __syncthreads();
+  for (int q = threadIdx.x; q < P * R2; q += blockDim.x) {
+    const int j0 = q % R2, r = q / R2;
+    const T* row = base + (size_t)r * N + j0;
+    Cx<T> x[R1];
+#pragma unroll
+    for (int m = 0; m < R1; ++m) x[m] = {row[m * R2], row[(size_t)P * N + m * R2]};
+    dft_r<T, R1>(x);
+#pragma unroll
+    for (int k1 = 0; k1 < R1; ++k1) S[r * LD + at(j0 + R2 * k1)] = k1 && j0 ? cmul(x[k1], tw[j0 * k1]) : x[k1];
+  }
+  __syncthreads();
+  if constexpr (R2 > 1) {
+    for (int q = threadIdx.x; q < P * R1; q += blockDim.x) {
+      Cx<T>* s = S + (q / R1) * LD + (q % R1) * (R2 + 1);
+      Cx<T> x[R2];
+#pragma unroll
+      for (int j = 0; j < R2; ++j) x[j] = s[j];
+      dft_r<T, R2>(x);
+#pragma unroll
+      for (int j = 0; j < R2; ++j) s[j] = x[j];
+    }
+    __syncthreads();
+  }
+  for (int q = threadIdx.x; q < P * (N / 2); q += blockDim.x) {
+    const int k = q % (N / 2), r = q / (N / 2), km = k ? N - k : N / 2;
+    const Cx<T> zk = S[r * LD + at((k % R1) * R2 + k / R1)], zm = S[r * LD + at((km % R1) * R2 + km / R1)];
+    const Sep<T> o = k ? separate(zk, zm) : separate_ends(zk, zm);
+    T* a = base + (size_t)r * N;
+    T* b = a + (size_t)P * N;
+    a[k] = (T)0.5 * o.ak;
+    b[k] = (T)0.5 * o.bk;
+    a[km] = (T)0.5 * o.am;
+    b[km] = (T)0.5 * o.bm;
+  }
+}
+// calls f with the radices of an n-point line as integral constants; false beyond 256 points
+template <class F>
+static bool with_radices(int n, F f) {
+  using std::integral_constant;
+  switch (n) {
+    case 4: f(integral_constant<int, 4>(), integral_constant<int, 1>()); return true;
+    case 8: f(integral_constant<int, 8>(), integral_constant<int, 1>()); return true;
+    case 16: f(integral_constant<int, 16>(), integral_constant<int, 1>()); return true;
+    case 32: f(integral_constant<int, 8>(), integral_constant<int, 4>()); return true;
+    case 64: f(integral_constant<int, 8>(), integral_constant<int, 8>()); return true;
+    case 128: f(integral_constant<int, 16>(), integral_constant<int, 8>()); return true;
+    case 256: f(integral_constant<int, 16>(), integral_constant<int, 16>()); return true;
+    default: return false;
+  }
+}
+static int dht1_threads(int P, int r) { return std::max(32, P * r); }
+// line pairs per block: 16 (whole 128-byte lines of FP64 columns), fewer where
+// that leaves under four blocks per SM
+static int dht1_pairs(long long pairs, int most) {
+  int P = std::min(DHT1_PAIRS, most);
+  while (P > 4 && pairs / P < 4 * 152) P /= 2;
+  return P;
+}
+
+// ---- FP32: both transforms of planes that fit one SM's shared memory, one CTA per plane
+// The separate kernels read and write the field twice per transform. Here a
+// CTA holds the plane as complex column pairs (c, c + nz/2) in shared memory
+// and every pass is an R-point DFT in registers, N = R1 R2, in place (a thread
+// stores to the slots it loaded), so both directions take four passes and
+// barriers:
+//   y1: from global memory, rows j0 + R2 m -> W^{j0 k1} -> rows j0 + R2 k1
+//   y2: rows k1 R2 + j0; wavenumber ky = k1 + R1 k2 ends at row k1 R2 + k2
+//   z1: the packed rows of the z transform are ky and ny - ky, so the
+//       separation of the y transform needs only Z_ky and Z_{ny-ky} of a
+//       column pair, both at hand; column position p < nz/2 of row pair
+//       (ky, ny - ky) lives in slot (row of ky, p), p >= nz/2 in (row of
+//       ny - ky, p - nz/2), which are the slots the thread read
+//   z2, then the separation of the row pairs on the way to global memory.
+// Columns are padded by one slot per R2 of the z direction (conflict-free
+// strides in z1, z2 and the last pass). Bound by shared memory and latency;
+// sizes are template parameters, because index arithmetic on run-time strides
+// cost a third of the time. 256 planes of 128 x 128: 0.072 (y, z) -> 0.014 ms.
+template <int R1Y, int R2Y, int R1Z, int R2Z>
+struct PlaneSize {
+  static constexpr int NY = R1Y * R2Y, NZ = R1Z * R2Z, NZH = NZ / 2;
+  static constexpr int LD = NZH + (R2Z > 1 ? NZH / R2Z : 0);
+  static constexpr int THREADS = NZH * R2Y < 64 ? 64 : NZH * R2Y > 512 ? 512 : NZH * R2Y;   // one item of y1 each
+  static constexpr size_t SMEM = ((size_t)NY * LD + NY + NZ) * sizeof(Cx<float>);
+  static constexpr bool FITS = SMEM <= 200 * 1024;
+};
+template <int R1Y, int R2Y, int R1Z, int R2Z>
+__global__ void __launch_bounds__((PlaneSize<R1Y, R2Y, R1Z, R2Z>::THREADS), (PlaneSize<R1Y, R2Y, R1Z, R2Z>::THREADS == 512 ? 2 : 1))
+k_dht2d_plane(const float* in, float* out, const float* __restrict__ twy, const float* __restrict__ twz) {
+  using G = PlaneSize<R1Y, R2Y, R1Z, R2Z>;
+  using C = Cx<float>;
+  constexpr int NY = G::NY, NZ = G::NZ, NZH = G::NZH, LD = G::LD, TH = G::THREADS;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  C* S = reinterpret_cast<C*>(smem_raw);
+  C* ty = S + NY * LD;
+  C* tz = ty + NY;
+  in += (size_t)blockIdx.x * NY * NZ;
+  out += (size_t)blockIdx.x * NY * NZ;
+  auto col = [](int c) { return R2Z > 1 ? c + c / R2Z : c; };
+  // row slots of wavenumber pair rp: ky = rp and ny - rp (0 and ny / 2 for rp = 0)
+  auto rows = [&](int rp, C*& a, C*& b) {
+    const int kb = rp ? NY - rp : NY / 2;
+    a = S + ((rp % R1Y) * R2Y + rp / R1Y) * LD;
+    b = S + ((kb % R1Y) * R2Y + kb / R1Y) * LD;
+  };
+  const int tid = threadIdx.x;
+  // the first pass's loads are issued before the twiddle tables are filled
+  for (int q0 = 0; q0 < NZH * R2Y; q0 += TH) {
+    const int q = q0 + tid, c = q % NZH, j0 = q / NZH;
+    const bool on = NZH * R2Y % TH == 0 || q < NZH * R2Y;
+    C x[R1Y];
+    if (on) {
+      const float* p = in + j0 * NZ + c;
+#pragma unroll
+      for (int m = 0; m < R1Y; ++m) x[m] = {__ldcg(p + m * R2Y * NZ), __ldcg(p + m * R2Y * NZ + NZH)};
+    }
+    if (q0 == 0) {
+      for (int t = tid; t < NY / 2; t += TH) {
+        ty[t] = {twy[2 * t], twy[2 * t + 1]};
+        ty[t + NY / 2] = {-twy[2 * t], -twy[2 * t + 1]};
+      }
+      for (int t = tid; t < NZ / 2; t += TH) {
+        tz[t] = {twz[2 * t], twz[2 * t + 1]};
+        tz[t + NZ / 2] = {-twz[2 * t], -twz[2 * t + 1]};
+      }
+      __syncthreads();
+    }
+    if (on) {
+      dft_r<float, R1Y>(x);
+      C* s = S + j0 * LD + col(c);
+#pragma unroll
+      for (int k1 = 0; k1 < R1Y; ++k1) s[k1 * R2Y * LD] = R2Y > 1 && k1 ? cmul(x[k1], ty[j0 * k1]) : x[k1];
+    }
+  }
+  __syncthreads();
+  if constexpr (R2Y > 1) {
+    for (int q = tid; q < NZH * R1Y; q += TH) {
+      C* s = S + (q / NZH) * R2Y * LD + col(q % NZH);
+      C x[R2Y];
+#pragma unroll
+      for (int j = 0; j < R2Y; ++j) x[j] = s[j * LD];
+      dft_r<float, R2Y>(x);
+#pragma unroll
+      for (int j = 0; j < R2Y; ++j) s[j * LD] = x[j];
+    }
+    __syncthreads();
+  }
+  for (int q = tid; q < (NY / 2) * R2Z; q += TH) {
+    const int j0 = q % R2Z, rp = q / R2Z;
+    C *a, *b;
+    rows(rp, a, b);
+    C x[R1Z];
+#pragma unroll
+    for (int m = 0; m < R1Z / 2; ++m) {
+      const int c = col(j0 + m * R2Z);
+      const C za = a[c], zb = b[c];
+      const Sep<float> o = rp ? separate(za, zb) : separate_ends(za, zb);
+      x[m] = {o.ak, o.am};              // column c of rows ky, ny - ky
+      x[m + R1Z / 2] = {o.bk, o.bm};    // column c + nz / 2
+    }
+    dft_r<float, R1Z>(x);
+#pragma unroll
+    for (int k1 = 0; k1 < R1Z; ++k1)
+      (k1 < R1Z / 2 ? a : b)[col(j0 + (k1 % (R1Z / 2)) * R2Z)] = R2Z > 1 && k1 ? cmul(x[k1], tz[j0 * k1]) : x[k1];
+  }
+  __syncthreads();
+  if constexpr (R2Z > 1) {
+    for (int q = tid; q < (NY / 2) * R1Z; q += TH) {
+      const int k1 = q % R1Z;
+      C *a, *b;
+      rows(q / R1Z, a, b);
+      C* s = (k1 < R1Z / 2 ? a : b) + (k1 % (R1Z / 2)) * (R2Z + 1);
+      C x[R2Z];
+#pragma unroll
+      for (int j = 0; j < R2Z; ++j) x[j] = s[j];
+      dft_r<float, R2Z>(x);
+#pragma unroll
+      for (int j = 0; j < R2Z; ++j) s[j] = x[j];
+    }
+    __syncthreads();
+  }
+  for (int q = tid; q < (NY / 2) * NZH; q += TH) {
+    const int k = q % NZH, rp = q / NZH, km = k ? NZ - k : NZH;
+    C *a, *b;
+    rows(rp, a, b);
+    const int pk = (k % R1Z) * R2Z + k / R1Z, pm = (km % R1Z) * R2Z + km / R1Z;
+    const C zk = (pk < NZH ? a : b)[col(pk % NZH)], zm = (pm < NZH ? a : b)[col(pm % NZH)];
+    const Sep<float> o = k ? separate(zk, zm) : separate_ends(zk, zm);
+    float* ra = out + rp * NZ;
+    float* rb = out + (rp ? NY - rp : NY / 2) * NZ;
+    ra[k] = 0.25f * o.ak;   // a half for each direction's separation
+    rb[k] = 0.25f * o.bk;
+    ra[km] = 0.25f * o.am;
+    rb[km] = 0.25f * o.bm;
+  }
+}
+// calls f with the PlaneSize of ny x nz planes; false where there is none that fits
+template <class F>
+static bool with_plane(int ny, int nz, F f) {
+  bool fits = false;
+  const bool known = with_radices(ny, [&](auto r1y, auto r2y) {
+    fits = with_radices(nz, [&](auto r1z, auto r2z) {
+      using G = PlaneSize<decltype(r1y)::value, decltype(r2y)::value, decltype(r1z)::value, decltype(r2z)::value>;
+      if constexpr (G::FITS)
+        f(G(), k_dht2d_plane<decltype(r1y)::value, decltype(r2y)::value, decltype(r1z)::value, decltype(r2z)::value>);
+    });
+  });
+  return known && fits && !(ny == 256 && nz == 256);
+}
+bool dht2d_plane_supported(int ny, int nz) {
+  return with_plane(ny, nz, [](auto, auto) {});
 }
 
 // Thomas solve along x per mode; rhs scaled by h^2 / (ny nz) (Hartley
@@ -902,12 +983,15 @@ __global__ void k_poisson_table(Consts c, T* __restrict__ tab, int* __restrict__
 
 template <class T>
 void launch_dht_y(const Consts& c, const Fields<T>& f, cudaStream_t s) {
-  if (c.ny == 256 && c.nz % 32 == 0) {
-    const size_t sh = (size_t)256 * 33 * sizeof(T) + 16 * WFFT_BUF * sizeof(Cx<T>);
-    k_dht_y256<T><<<c.nx * (c.nz / 32), 512, sh, s>>>(f.phi, c.nz, f.tw_y);
+  const int n = c.ny;
+  if (with_radices(n, [&](auto r1, auto r2) {
+        constexpr int R1 = decltype(r1)::value, R2 = decltype(r2)::value;
+        const int P = dht1_pairs((long long)c.nx * c.nz / 2, c.nz / 2);
+        const size_t sh = (size_t)R1 * R2 * (P + 1) * sizeof(Cx<T>);
+        k_dht1_y<T, R1, R2><<<c.nx * (c.nz / (2 * P)), dht1_threads(P, std::max(R1, R2)), sh, s>>>(f.phi, c.nz, P, f.tw_y);
+      }))
     return;
-  }
-  const int n = c.ny, logn = (int)std::lround(std::log2((double)n));
+  const int logn = (int)std::lround(std::log2((double)n));
   const int W = c.nz < 16 ? c.nz : 16;
   const size_t sh = (size_t)(W / 2) * n * sizeof(typename Vec2<T>::type);
   // group = one x plane; lines = nz columns; positions nz apart
@@ -917,12 +1001,15 @@ void launch_dht_y(const Consts& c, const Fields<T>& f, cudaStream_t s) {
 
 template <class T>
 void launch_dht_z(const Consts& c, const Fields<T>& f, cudaStream_t s) {
-  if (c.nz == 256) {
-    const int rows = c.nx * c.ny;   // even: ny is an even power of two
-    k_dht_z256<T><<<(rows / 2 + 7) / 8, 256, 0, s>>>(f.phi, rows, f.tw_z);
+  const int n = c.nz;
+  if (with_radices(n, [&](auto r1, auto r2) {
+        constexpr int R1 = decltype(r1)::value, R2 = decltype(r2)::value;
+        const int P = dht1_pairs((long long)c.nx * c.ny / 2, c.ny / 2);
+        const size_t sh = ((size_t)(R1 * R2 + (R2 > 1 ? R1 : 1)) * P + R1 * R2) * sizeof(Cx<T>);
+        k_dht1_z<T, R1, R2><<<c.nx * (c.ny / (2 * P)), dht1_threads(P, std::max(R1, R2)), sh, s>>>(f.phi, P, f.tw_z);
+      }))
     return;
-  }
-  const int n = c.nz, logn = (int)std::lround(std::log2((double)n));
+  const int logn = (int)std::lround(std::log2((double)n));
   const int lines = c.nx * c.ny;
   int W = 16;
   while (lines % W) W >>= 1;   // ny is an even power of two, so W >= 2
@@ -953,22 +1040,24 @@ void launch_poisson_x(const Consts& c, const Fields<T>& f, cudaStream_t s) {
   launch_poisson_x_on(c, f, f.phi, s);
 }
 
-template <class T>
-bool launch_dht2d(const Consts& c, const Fields<T>& f, cudaStream_t s) {
-  if (c.ny != 256 || c.nz != 256) return false;
-  if constexpr (sizeof(T) == 4) {
-    k_dht2d_r16<<<c.nx * R16_CLUSTER, R16_THREADS, R16_SMEM, s>>>(f.phi, f.phi, f.tw_y);
+// FP32: both transforms of every x plane in one pass where a kernel has the
+// shape, 256 x 256 in clusters, planes that fit shared memory one CTA each. FP64
+// takes the directions one by one: its pipe bounds them either way, and the
+// small blocks of k_dht1_y, k_dht1_z fill the SMs evenly (512 planes of 256 x
+// 256: 2.06 ms in the cluster form, 1.88 here)
+bool launch_dht2d_on(const Consts& c, const Fields<float>& f, const float* in, float* out, cudaStream_t s) {
+  if (c.ny == 256 && c.nz == 256) {
+    k_dht2d_r16<<<c.nx * R16_CLUSTER, R16_THREADS, R16_SMEM, s>>>(in, out, f.tw_y);
     return true;
   }
-  const size_t sh = (size_t)256 * 33 * sizeof(T) + (DHT2D_THREADS / 32) * WFFT_BUF * sizeof(Cx<T>);
-  k_dht2d_256<T><<<c.nx * DHT2D_CLUSTER, DHT2D_THREADS, sh, s>>>(f.phi, f.tw_y);
-  return true;
+  return with_plane(c.ny, c.nz, [&](auto g, auto kernel) {
+    kernel<<<c.nx, decltype(g)::THREADS, decltype(g)::SMEM, s>>>(in, out, f.tw_y, f.tw_z);
+  });
 }
-
-bool launch_dht2d_on(const Consts& c, const Fields<float>& f, const float* in, float* out, cudaStream_t s) {
-  if (c.ny != 256 || c.nz != 256) return false;
-  k_dht2d_r16<<<c.nx * R16_CLUSTER, R16_THREADS, R16_SMEM, s>>>(in, out, f.tw_y);
-  return true;
+template <class T>
+bool launch_dht2d(const Consts& c, const Fields<T>& f, cudaStream_t s) {
+  if constexpr (sizeof(T) == 4) return launch_dht2d_on(c, f, f.phi, f.phi, s);
+  else return false;
 }
 
 // the same transform of `nplanes` 256 x 256 planes outside a solver state
@@ -1019,11 +1108,20 @@ template void launch_poisson_table<float>(const Consts&, const Fields<float>&, c
 
 // opt in to large dynamic shared memory for the transform kernels
 void poisson_set_attributes() {
-  cudaFuncSetAttribute(k_dht2d_256<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-  cudaFuncSetAttribute(k_dht2d_256<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
   cudaFuncSetAttribute(k_dht2d_r16, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)R16_SMEM);
-  cudaFuncSetAttribute(k_dht_y256<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-  cudaFuncSetAttribute(k_dht_y256<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+  for (int n = 4; n <= 256; n *= 2) {
+    for (int m = 4; m <= 256; m *= 2)
+      with_plane(n, m, [](auto g, auto kernel) {
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)decltype(g)::SMEM);
+      });
+    with_radices(n, [](auto r1, auto r2) {
+      constexpr int R1 = decltype(r1)::value, R2 = decltype(r2)::value;
+      cudaFuncSetAttribute(k_dht1_y<double, R1, R2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
+      cudaFuncSetAttribute(k_dht1_z<double, R1, R2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
+      cudaFuncSetAttribute(k_dht1_y<float, R1, R2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
+      cudaFuncSetAttribute(k_dht1_z<float, R1, R2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
+    });
+  }
   cudaFuncSetAttribute(k_dht<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
   cudaFuncSetAttribute(k_dht<double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
   cudaFuncSetAttribute(k_dht<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);

@@ -140,7 +140,9 @@ template <class T> void launch_af_y(const Consts& c, const Fields<T>& f, int cur
 template <class T> void launch_af_z(const Consts& c, const Fields<T>& f, int cur, cudaStream_t s);
 template <class T> bool launch_af_yz(const Consts& c, const Fields<T>& f, int cur, cudaStream_t s);
 template <class T> bool launch_dht2d(const Consts& c, const Fields<T>& f, cudaStream_t s);
-// FP32 2-D transform of every 256 x 256 plane from `in` to `out` (may alias); false for other shapes
+// FP32 2-D transform of every x plane from `in` to `out` (may alias); false for planes neither
+// 256 x 256 nor small enough for one SM's shared memory (dht2d_plane_supported)
+bool dht2d_plane_supported(int ny, int nz);
 bool launch_dht2d_on(const Consts& c, const Fields<float>& f, const float* in, float* out, cudaStream_t s);
 bool dht2d_planes_fp32(const float* in, float* out, int nplanes, const float* tw, cudaStream_t s);
 template <class T> void launch_mass(const Consts& c, const Fields<T>& f, int cur, cudaStream_t s);
