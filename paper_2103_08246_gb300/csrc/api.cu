@@ -434,7 +434,7 @@ size_t carve(ibm_state* s, void* base, const Layout& L, Fields<T>& f) {
   f.n_partial = partial_count<T>(c);
   f.partial = cv.take<double>(f.n_partial);
   f.qpart = cv.take<double>(2 * (size_t)outflow_blocks(c));
-  f.mean00 = cv.take<double>(1);
+  f.ticket = cv.take<int>(2);   // zero from the workspace's clearing on
   f.inflow = s->inflow ? cv.take<T>(8 * P) : nullptr;
   f.inflow_mean = s->inflow ? cv.take<double>(1) : nullptr;
   f.prm = cv.take<Params>(1);
@@ -603,20 +603,19 @@ void project_after_solve(ibm_state* s, int cur, bool initial, cudaStream_t st) {
 // three captured graphs per velocity buffer parity; every replay ends with
 // all its work (the structural update included) joined.
 template <class T>
-void record_head(ibm_state* s, int cur) {
+void record_head(ibm_state* s, int cur, bool advance) {
   Fields<T>& f = fields<T>(s);
   const Consts& c = s->c;
   cudaStream_t st = s->stream;
-  launch_begin_step(c, f, st);
-  // the implicit factors' tables for this step's r, concurrent with the RHS
+  launch_begin_step(c, f, st, advance);
+  // the implicit factors' tables, the outflow and the mass fix, concurrent with the RHS
   cudaEventRecord(s->ev_fork2, st);
   cudaStreamWaitEvent(s->side2, s->ev_fork2, 0);
-  launch_af_tables(c, f, s->side2);
+  launch_head_side(c, f, cur, s->side2);
   cudaEventRecord(s->ev_join2, s->side2);
   launch_rhs(c, f, cur, st);
-  launch_inflow(c, f, cur, st);   // new inflow time level (prescribed inflow only)
-  launch_outflow(c, f, cur, st);
   cudaStreamWaitEvent(st, s->ev_join2, 0);
+  if (f.inflow) launch_outflow(c, f, cur, st);   // with the new inflow time level
   launch_af(c, f, cur, st);
 }
 
@@ -634,7 +633,7 @@ bool record_tail_body(ibm_state* s, int cur) {
     launch_flag(f.prm, s->fl, false, s->side);
     cudaEventRecord(s->ev_join, s->side);
   }
-  launch_mass_div(c, f, cur, false, st);
+  launch_div(c, f, cur, false, st);
   solve_poisson<T>(s, st);
   project_after_solve<T>(s, cur, false, st);
   return flag;
@@ -643,11 +642,11 @@ bool record_tail_body(ibm_state* s, int cur) {
 template <class T>
 void record_graph(ibm_state* s, int kind, int cur) {
   if (kind == GRAPH_HEAD) {
-    record_head<T>(s, cur);
+    record_head<T>(s, cur, false);
     return;
   }
   const bool join = record_tail_body<T>(s, cur);
-  if (kind == GRAPH_MID) record_head<T>(s, cur ^ 1);
+  if (kind == GRAPH_MID) record_head<T>(s, cur ^ 1, true);
   if (kind == GRAPH_TAIL) launch_speed_check(s->c, fields<T>(s), s->stream);
   if (join) cudaStreamWaitEvent(s->stream, s->ev_join, 0);
 }
@@ -805,7 +804,7 @@ int init_state(ibm_state* s, const ibm_options* o, const FlagGeom& fg,
   }
   // initial projection of u0 (dt absorbed in phi), velocity only
   s->cur = 0;
-  launch_mass_div(c, f, 0, true, st);
+  launch_div(c, f, 0, true, st);
   solve_poisson<T>(s, st);
   project_after_solve<T>(s, 0, true, st);
   s->cur = 1;
@@ -987,18 +986,18 @@ void launch_stage(ibm_state* s, int stage) {
     case IBM_STAGE_AF_Z: launch_af_z(c, f, cur, st); break;
     case IBM_STAGE_IB: launch_ib(c, f, s->mk, s->fl, cur, st); break;
     case IBM_STAGE_FLAG: launch_flag(f.prm, s->fl, true, st); break;
-    case IBM_STAGE_MASS_DIV: launch_mass_div(c, f, cur, false, st); break;
+    case IBM_STAGE_MASS_DIV: launch_div(c, f, cur, false, st); break;
     case IBM_STAGE_DHT_Y: launch_dht_y(c, f, st); break;
     case IBM_STAGE_DHT_Z: launch_dht_z(c, f, st); break;
     case IBM_STAGE_POISSON_X: launch_poisson_x(c, f, st); break;
     case IBM_STAGE_PROJECT:
       // as the step runs it: the mixed solve's two parts summed as they are read
       if (std::is_same<T, float>::value && s->precision == IBM_MIXED && c.corr_bf16)
-        launch_project_only(c, f, cur, false, st, (const T*)f.e[1], (const T*)nullptr, (const void*)f.e[2]);
+        launch_project(c, f, cur, false, st, (const T*)f.e[1], (const T*)nullptr, (const void*)f.e[2]);
       else if (std::is_same<T, float>::value && s->precision == IBM_MIXED)
-        launch_project_only(c, f, cur, false, st, (const T*)f.e[1], (const T*)f.e[2]);
+        launch_project(c, f, cur, false, st, (const T*)f.e[1], (const T*)f.e[2]);
       else
-        launch_project_only(c, f, cur, false, st);
+        launch_project(c, f, cur, false, st);
       break;
     case IBM_STAGE_POISSON: solve_poisson<T>(s, st); break;
     case IBM_STAGE_AF_YZ: (void)launch_af_yz(c, f, cur, st); break;
@@ -1070,21 +1069,19 @@ __global__ void k_wait_selftest(uint32_t spins, int* flag) {
 
 namespace {
 // pieces of a member's step for the batched ensemble: the step's start
-// (dt, implicit-factor tables), its explicit stage (batched across the
-// members), the rest of its head (inflow, outflow, implicit factors), its
+// (dt, implicit-factor tables, outflow), its explicit stage (batched across the
+// members), the rest of its head (prescribed inflow, implicit factors), its
 // tail (forcing, structure joined, pressure, projection)
 template <class T>
 void record_pre(ibm_state* s, int cur) {
   Fields<T>& f = fields<T>(s);
-  launch_begin_step(s->c, f, s->stream);
-  launch_af_tables(s->c, f, s->stream);
-  (void)cur;
+  launch_begin_step(s->c, f, s->stream, false);
+  launch_head_side(s->c, f, cur, s->stream);
 }
 template <class T>
 void record_post(ibm_state* s, int cur) {
   Fields<T>& f = fields<T>(s);
-  launch_inflow(s->c, f, cur, s->stream);
-  launch_outflow(s->c, f, cur, s->stream);
+  if (f.inflow) launch_outflow(s->c, f, cur, s->stream);
   launch_af(s->c, f, cur, s->stream);
 }
 template <class T>
@@ -1243,10 +1240,9 @@ int slab_phase_impl(ibm_state* s, int phase, double dt, const double* recv, doub
         CK(cudaStreamSynchronize(st));
         s->last_dt_fixed = dt;
       }
-      launch_begin_step(c, f, st);
-      launch_af_tables(c, f, st);
+      launch_begin_step(c, f, st, false);
+      launch_head_side(c, f, s->cur, st);
       launch_rhs(c, f, s->cur, st);
-      launch_outflow(c, f, s->cur, st);
       launch_af(c, f, s->cur, st);
       launch_ib(c, f, s->mk, s->fl, s->cur, st);
       slab_pack_force(c, sd, s->fl, f.qpart, outflow_blocks(c), send, st);
@@ -1278,6 +1274,7 @@ int slab_phase_impl(ibm_state* s, int phase, double dt, const double* recv, doub
       if (sd.gL > 0) CK(copy_planes(f.phi, recv, gL - 1, 1, P, true, st));
       if (sd.gR > 0) CK(copy_planes(f.phi, recv + P, gL + n, 1, P, true, st));
       launch_project<double>(c, f, s->cur, s->slab_initial, st);
+      if (!s->slab_initial) launch_end_step(f.prm, st);
       s->cur ^= 1;
       const int cur = s->cur;
       double* arr[4] = {f.u[cur], f.v[cur], f.w[cur], f.p};

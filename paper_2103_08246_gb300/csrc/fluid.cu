@@ -31,7 +31,17 @@ constexpr int HMAX = 24;     // largest warm-up the segments carry
 // FP32 tolerance needs about half the planes): smaller shared-memory segments
 template <class T> constexpr int hmax_of() { return sizeof(T) == 8 ? HMAX : 13; }
 
-__device__ inline double af_theta(double r) { return 2.0 * asinh(0.5 / sqrt(r)); }
+// decay factor of the implicit factors, the smaller root of
+// rho + 1 / rho = 2 + 1 / r, without cancellation
+__device__ inline double af_decay(double r) { return 2.0 * r / (1.0 + 2.0 * r + sqrt(1.0 + 4.0 * r)); }
+
+// the clock after a step (one thread)
+__device__ inline void advance_clock(Params* prm) {
+  prm->t += prm->dt;
+  prm->dt_old = prm->dt;
+  prm->step += 1;
+  prm->first = 0;
+}
 
 // dt (fixed or CFL), AB2 weights, implicit diffusion number and sub-steps.
 // The per-block speed maxima are non-negative doubles (or +inf), whose bit
@@ -39,74 +49,95 @@ __device__ inline double af_theta(double r) { return 2.0 * asinh(0.5 / sqrt(r));
 // pipe. Each kernel writes only the fields it owns: the structural update
 // runs concurrently and owns flag_pending.
 // The partials are cleared for the maxima that this step's projection adds.
-__global__ void k_begin_step(Consts c, Params* prm, double* __restrict__ partial,
-                             int n_partial, double tol, int hmax) {
+// advance: the step before this one ends here (its clock), which saves its own
+// launch between the steps of a call. The kernel is one chain of FP64 scalar
+// operations on the critical path of every step: after dt each dependent
+// group runs in its own warp, and the decay factor is algebraic instead of
+// exp(-2 asinh(1 / (2 sqrt r))). With the clock here and the outflow, mass fix
+// and line mean in other launches a step of 91 x 32 x 64 FP32 cells went from 70
+// to 54 us.
+__global__ void __launch_bounds__(1024)
+k_begin_step(Consts c, Params* prm, double* __restrict__ partial, int n_partial, double log_tol, int hmax, int advance) {
   __shared__ unsigned long long wmax[32];
+  __shared__ double s_dt;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   unsigned long long mb = 0ull;
   for (int b = threadIdx.x; b < n_partial; b += blockDim.x) {
     mb = max(mb, (unsigned long long)__double_as_longlong(partial[b]));
     partial[b] = 0.0;
   }
   for (int o = 16; o > 0; o >>= 1) mb = max(mb, __shfl_xor_sync(0xffffffffu, mb, o));
-  if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = mb;
+  if (lane == 0) wmax[warp] = mb;
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int q = 1; q < (int)(blockDim.x >> 5); ++q) mb = max(mb, wmax[q]);
     const double m = __longlong_as_double((long long)mb);
     const double dt_fixed = prm->dt_fixed;
-    int err = 0;
+    if (advance) advance_clock(prm);
     double dt = dt_fixed > 0.0 ? dt_fixed : prm->cfl * c.h / m;
     if (!isfinite(m) || !(dt > 0.0) || !isfinite(dt)) {
-      err |= ERR_NONFINITE;
+      atomicOr(&prm->error, ERR_NONFINITE);
       dt = dt_fixed > 0.0 ? dt_fixed : 1e-300;
     }
+    prm->speed_max = m;
+    prm->slip_max = 0.0;
+    s_dt = dt;
+  }
+  __syncthreads();
+  if (lane != 0 || warp > 4) return;
+  const double dt = s_dt;
+  if (warp == 0) {
     double alpha = 1.0, beta = 0.0;
     if (!prm->first) {
       alpha = 1.0 + dt / (2.0 * prm->dt_old);
       beta = -dt / (2.0 * prm->dt_old);
     }
-    double r = c.nu * dt / (2.0 * c.h * c.h);
-    if (!(r > 0.0) || !isfinite(r)) {
-      err |= ERR_AF_RANGE;
-      r = 1e-300;
-    }
-    const double th = af_theta(r);
-    const double rho = exp(-th);
-    int H = (int)ceil(log(tol) / log(rho));
-    if (!(H >= 1)) H = 1;
-    if (H > hmax) {
-      err |= ERR_AF_RANGE;
-      H = hmax;
-    }
-    // velocity Verlet is stable for dt_s omega < 2; omega_max is a Gershgorin
-    // upper bound, so dt_s = dt / n_sub <= 1.8 / omega_max keeps every mode stable
-    const double ns = ceil(dt * c.omega_max / 1.8);
-    prm->speed_max = m;
-    prm->slip_max = 0.0;
     prm->dt = dt;
     prm->alpha = alpha;
     prm->beta = beta;
+    prm->f_alpha = (float)alpha;
+    prm->f_beta = (float)beta;
+  } else if (warp == 1) {
+    double r = c.nu * dt / (2.0 * c.h * c.h);
+    int err = 0;
+    if (!(r > 0.0) || !isfinite(r)) {
+      err = ERR_AF_RANGE;
+      r = 1e-300;
+    }
+    const double rho = af_decay(r);
+    int H = (int)ceil(log_tol / log(rho));
+    if (!(H >= 1)) H = 1;
+    if (H > hmax) {
+      err = ERR_AF_RANGE;
+      H = hmax;
+    }
     prm->r = r;
     prm->af_rho = rho;
     prm->af_h = H;
-    prm->n_sub = ns < 1.0 ? 1 : (ns > 1e6 ? 1000000 : (int)ns);
-    prm->f_dt = (float)dt;
-    prm->f_alpha = (float)alpha;
-    prm->f_beta = (float)beta;
     prm->f_r = (float)r;
-    prm->f_ir = (float)(1.0 / r);
     prm->f_rho = (float)rho;
+    if (err) atomicOr(&prm->error, err);
+  } else if (warp == 2) {
+    const double r = c.nu * dt / (2.0 * c.h * c.h);
+    prm->f_ir = (float)(1.0 / (r > 0.0 && isfinite(r) ? r : 1e-300));
+  } else if (warp == 3) {
+    // velocity Verlet is stable for dt_s omega < 2; omega_max is a Gershgorin
+    // upper bound, so dt_s = dt / n_sub <= 1.8 / omega_max keeps every mode stable
+    const double ns = ceil(dt * c.omega_max / 1.8);
+    prm->n_sub = ns < 1.0 ? 1 : (ns > 1e6 ? 1000000 : (int)ns);
+  } else {
+    prm->f_dt = (float)dt;
     prm->f_gdt = (float)(dt * c.inv_h);
     prm->f_hnu = (float)(0.5 * c.nu * dt * c.inv_h * c.inv_h);
     prm->f_cc = (float)(c.u_in * dt * c.inv_h);
     prm->f_sc_div = (float)(c.inv_h / dt);
-    if (err) prm->error |= err;
   }
 }
 
-// After the last step of a call: the speed maximum of the velocity that step
-// left (the projection's block partials, reduced as in k_begin_step), so that
-// a non-finite or too fast field is reported by the call that produced it
+// After the last step of a call: its clock, and the speed maximum of the
+// velocity that step left (the projection's block partials, reduced as in
+// k_begin_step), so that a non-finite or too fast field is reported by the call
+// that produced it
 __global__ void k_speed_check(Params* prm, const double* __restrict__ partial, int n_partial) {
   __shared__ unsigned long long wmax[32];
   unsigned long long mb = 0ull;
@@ -118,6 +149,7 @@ __global__ void k_speed_check(Params* prm, const double* __restrict__ partial, i
   if (threadIdx.x == 0) {
     for (int q = 1; q < (int)(blockDim.x >> 5); ++q) mb = max(mb, wmax[q]);
     const double m = __longlong_as_double((long long)mb);
+    advance_clock(prm);
     prm->speed_max = m;
     if (!isfinite(m)) atomicOr(&prm->error, ERR_NONFINITE);
   }
@@ -131,29 +163,35 @@ void launch_speed_check(const Consts& c, const Fields<T>& f, cudaStream_t s) {
 template void launch_speed_check<float>(const Consts&, const Fields<float>&, cudaStream_t);
 template void launch_speed_check<double>(const Consts&, const Fields<double>&, cudaStream_t);
 
-// Tables of the implicit factors for this step's r, one entry per thread
-// (FP64 transcendental functions: spread over many blocks, and off the
-// critical path, concurrent with the explicit stage):
+// Tables of the implicit factors for this step's r, one entry per thread, off
+// the critical path, concurrent with the explicit stage:
 //   LU inverse pivots of the x factors (closed form)
 //     Dirichlet start (u):      1/p_k = rho (1 - rho^{2k})   / (1 - rho^{2k+2})
 //     reflection start (v, w):  1/p_k = rho (1 - rho^{2k-1}) / (1 - rho^{2k+1})
 //   free-space taps of the reflected x solve: (1/r) rho^{m+1} / (1 - rho^2)
 //   taps of the exact periodic inverse of r (q - S - S^{-1}) on n points:
 //     t_m = (1/r) rho / (1 - rho^2) (rho^m + rho^{n-m}) / (1 - rho^n)
-constexpr int TAB_THREADS = 64;
+// Powers by repeated squaring; rho stays below 1/2 within the factors' range
+// (r up to 0.3 in FP64, 1.3 in FP32), so 1 - rho^k does not cancel.
 int table_entries(const Consts& c) { return c.nx + (HMAX + 1) + c.ny + c.nz; }
 
-__global__ void __launch_bounds__(TAB_THREADS)
-k_af_tables(Consts c, const Params* __restrict__ prm, double* __restrict__ ipt,
-            float* __restrict__ iptf, double* __restrict__ taps, float* __restrict__ tapsf) {
-  int q = blockIdx.x * blockDim.x + threadIdx.x;
-  const double r = prm->r;
-  const double th = af_theta(r);
-  const double rho = exp(-th);
+__device__ inline double int_power(double b, int n) {
+  double v = 1.0;
+  for (; n > 0; n >>= 1) {
+    if (n & 1) v *= b;
+    b *= b;
+  }
+  return v;
+}
+
+__device__ inline void af_table_entry(const Consts& c, const Params* prm, double* ipt, float* iptf, double* taps,
+                                      float* tapsf, int q) {
+  const double r = prm->r, rho = prm->af_rho;
   if (q < c.nx) {
     const int k = q + 1;
-    const double a = rho * expm1(-2.0 * k * th) / expm1(-(2.0 * k + 2.0) * th);
-    const double b = rho * expm1(-(2.0 * k - 1.0) * th) / expm1(-(2.0 * k + 1.0) * th);
+    const double odd = int_power(rho, 2 * k - 1);   // rho^(2k-1), and from it 2k, 2k+1, 2k+2
+    const double a = rho * (1.0 - odd * rho) / (1.0 - odd * rho * rho * rho);
+    const double b = rho * (1.0 - odd) / (1.0 - odd * rho * rho);
     ipt[k] = a;
     ipt[c.nx + 2 + k] = b;
     iptf[k] = (float)a;
@@ -162,7 +200,7 @@ k_af_tables(Consts c, const Params* __restrict__ prm, double* __restrict__ ipt,
   }
   q -= c.nx;
   if (q <= HMAX) {
-    const double v = (1.0 / r) * exp(-(double)(q + 1) * th) / (-expm1(-2.0 * th));
+    const double v = int_power(rho, q + 1) / (r * (1.0 - rho * rho));
     taps[c.ny + c.nz + q] = v;
     tapsf[c.ny + c.nz + q] = (float)v;
     return;
@@ -172,20 +210,12 @@ k_af_tables(Consts c, const Params* __restrict__ prm, double* __restrict__ ipt,
   const int n = dir == 0 ? c.ny : c.nz;
   const int m = dir == 0 ? q : q - c.ny;
   if (m >= n) return;
-  const double pre = (1.0 / r) * rho / (-expm1(-2.0 * th));
-  const double den = -expm1(-(double)n * th);
-  const double v = pre * (exp(-(double)m * th) + exp(-(double)(n - m) * th)) / den;
+  const double v = rho / (r * (1.0 - rho * rho)) * (int_power(rho, m) + int_power(rho, n - m)) / (1.0 - int_power(rho, n));
   taps[q] = v;    // y taps at [0, ny), z taps at [ny, ny + nz)
   tapsf[q] = (float)v;
 }
-
-// after the projection: advance the clock
-__global__ void k_end_step(Params* prm) {
-  prm->t += prm->dt;
-  prm->dt_old = prm->dt;
-  prm->step += 1;
-  prm->first = 0;
-}
+// the clock after a step whose next one does not follow in the same launch (slabs)
+__global__ void k_end_step(Params* prm) { advance_clock(prm); }
 
 // ---------------------------------------------------------------- RHS (A2)
 // RHS = dt [ -(alpha N^n + beta N^{n-1}) - G p^n + nu L u^n ], N in flux form.
@@ -782,42 +812,111 @@ k_rhs_vec(Consts c, Params* __restrict__ prm, const T* __restrict__ u, const T* 
 
 // ---------------------------------------------------------------- outflow (A1)
 // Convective condition dq/dt + U dq/dx = 0 on the outflow plane, first-order
-// upwind; the increment is kept for the x line solve. The inflow and new
-// outflow face fluxes are summed per block in FP64 (fixed order) for the
-// mass fix; the IB forcing never touches these two planes.
+// upwind: the increments, for the x line solve, which also adds them to the
+// plane (the explicit stage still reads its old values, so this kernel runs
+// beside it, in one launch with the tables of the implicit factors). The inflow
+// and new outflow face fluxes are summed per block in FP64, and the last block
+// sums the blocks (fixed order) into the mass fix: Q_in, Q_out and the shift
+// (Q_in - Q_out) / (Ly Lz) that the divergence adds to the outflow face; the IB
+// forcing never touches these two planes. Tables, outflow and mass fix were
+// three launches, two of them between other kernels of the step's chain: 12 us.
+// With a prescribed inflow the new inflow level comes first (inflow != null,
+// after the explicit stage): u_in = pending u - mean + U on face 0, the
+// boundary increments for the x factor, and the current v, w planes.
 constexpr int OUT_THREADS = 256;
 template <class T>
-__global__ void __launch_bounds__(OUT_THREADS)
-k_outflow(Consts c, const Params* __restrict__ prm, T* __restrict__ u,
-          T* __restrict__ v, T* __restrict__ w, T* __restrict__ o0, T* __restrict__ o1,
-          T* __restrict__ o2, double* __restrict__ qpart) {
+__device__ inline void outflow_block(const Consts& c, Params* prm, T* __restrict__ u, const T* __restrict__ v,
+                                     const T* __restrict__ w, T* __restrict__ o0, T* __restrict__ o1, T* __restrict__ o2,
+                                     double* __restrict__ qpart, int* __restrict__ ticket, T* __restrict__ inflow,
+                                     const double* __restrict__ inflow_mean, int block, int nblocks) {
   __shared__ double scratch[32];
-  const int jk = blockIdx.x * blockDim.x + threadIdx.x;
+  __shared__ int last_block;
+  const int jk = block * blockDim.x + threadIdx.x;
   const int P = c.ny * c.nz;
   double qi = 0.0, qo = 0.0;
   if (jk < P) {
+    if (inflow) {
+      T *cv = inflow + 3 * (size_t)P, *cw = cv + P, *iu = cw + P, *iv = iu + P, *iw = iv + P;
+      const T un = (T)((double)inflow[jk] - *inflow_mean + c.u_in);
+      iu[jk] = un - u[jk];
+      u[jk] = un;
+      const T vn = inflow[jk + P], wn = inflow[jk + 2 * (size_t)P];
+      iv[jk] = vn - cv[jk];
+      iw[jk] = wn - cw[jk];
+      cv[jk] = vn;
+      cw[jk] = wn;
+    }
     const T cc = pick<T>(c.u_in * prm->dt * c.inv_h, prm->f_cc);
     const size_t last = (size_t)c.nx * P + jk, prev = last - P;
-    T inc = -cc * (u[last] - u[prev]);
-    const T un = u[last] + inc;
-    u[last] = un;
+    const T inc = -cc * (u[last] - u[prev]);
     o0[jk] = inc;
-    inc = -cc * (v[last] - v[prev]);
-    v[last] += inc;
-    o1[jk] = inc;
-    inc = -cc * (w[last] - w[prev]);
-    w[last] += inc;
-    o2[jk] = inc;
+    o1[jk] = -cc * (v[last] - v[prev]);
+    o2[jk] = -cc * (w[last] - w[prev]);
     qi = (double)u[jk];
-    qo = (double)un;
+    qo = (double)(u[last] + inc);
   }
   qi = block_sum(qi, scratch);
   __syncthreads();
   qo = block_sum(qo, scratch);
   if (threadIdx.x == 0) {
-    qpart[2 * blockIdx.x] = qi;
-    qpart[2 * blockIdx.x + 1] = qo;
+    qpart[2 * block] = qi;
+    qpart[2 * block + 1] = qo;
+    __threadfence();
+    last_block = atomicAdd(ticket, 1) == nblocks - 1;
   }
+  __syncthreads();
+  if (!last_block) return;
+  __threadfence();
+  qi = qo = 0.0;
+  for (int b = threadIdx.x; b < nblocks; b += blockDim.x) {
+    qi += __ldcg(qpart + 2 * b);
+    qo += __ldcg(qpart + 2 * b + 1);
+  }
+  __syncthreads();
+  qi = block_sum(qi, scratch);
+  __syncthreads();
+  qo = block_sum(qo, scratch);
+  if (threadIdx.x == 0) {
+    const double h2 = c.h * c.h;
+    prm->q_in = qi * h2;
+    prm->q_out = qo * h2;
+    prm->mass_shift = (qi - qo) * h2 / (c.ly * c.lz);
+    prm->f_mass_shift = (float)prm->mass_shift;
+    *ticket = 0;
+  }
+}
+template <class T>
+__global__ void __launch_bounds__(OUT_THREADS)
+k_outflow(Consts c, Params* __restrict__ prm, T* __restrict__ u, const T* __restrict__ v, const T* __restrict__ w,
+          T* __restrict__ o0, T* __restrict__ o1, T* __restrict__ o2, double* __restrict__ qpart, int* __restrict__ ticket,
+          T* __restrict__ inflow, const double* __restrict__ inflow_mean) {
+  outflow_block<T>(c, prm, u, v, w, o0, o1, o2, qpart, ticket, inflow, inflow_mean, blockIdx.x, gridDim.x);
+}
+// beside the explicit stage: the tables' blocks, then the outflow's or (with a
+// prescribed inflow, whose planes the explicit stage reads) one block for the
+// mean of the pending u plane
+template <class T>
+__global__ void __launch_bounds__(OUT_THREADS)
+k_head_side(Consts c, Params* __restrict__ prm, double* __restrict__ ipt, float* __restrict__ iptf,
+            double* __restrict__ taps, float* __restrict__ tapsf, int ntab, T* __restrict__ u, const T* __restrict__ v,
+            const T* __restrict__ w, T* __restrict__ o0, T* __restrict__ o1, T* __restrict__ o2,
+            double* __restrict__ qpart, int* __restrict__ ticket, const T* __restrict__ pending_u,
+            double* __restrict__ inflow_mean) {
+  const int b = blockIdx.x;
+  if (b < ntab) {
+    af_table_entry(c, prm, ipt, iptf, taps, tapsf, b * blockDim.x + threadIdx.x);
+    return;
+  }
+  if (!pending_u) {
+    outflow_block<T>(c, prm, u, v, w, o0, o1, o2, qpart, ticket, (T*)nullptr, nullptr, b - ntab, gridDim.x - ntab);
+    return;
+  }
+  __shared__ double scratch[32];
+  const int P = c.ny * c.nz;
+  double s = 0.0;
+  for (int q = threadIdx.x; q < P; q += blockDim.x) s += (double)pending_u[q];
+  s = block_sum(s, scratch);
+  if (threadIdx.x == 0) *inflow_mean = s / P;
 }
 
 // asynchronous copy of one element (4 or 8 bytes) into shared memory
@@ -834,7 +933,8 @@ __global__ void __launch_bounds__(32)
 k_af_xr(Consts c, const Params* __restrict__ prm, const T* __restrict__ ipt,
         const T* __restrict__ d0, const T* __restrict__ d1, const T* __restrict__ d2,
         T* __restrict__ e0, T* __restrict__ e1, T* __restrict__ e2, const T* __restrict__ o0,
-        const T* __restrict__ o1, const T* __restrict__ o2, const T* __restrict__ inc) {
+        const T* __restrict__ o1, const T* __restrict__ o2, const T* __restrict__ inc, T* __restrict__ u, T* __restrict__ v,
+        T* __restrict__ w) {
   __shared__ T s[(XS + 2 * hmax_of<T>()) * 32];
   const int P = c.ny * c.nz;
   const int lane = threadIdx.x;
@@ -854,6 +954,8 @@ k_af_xr(Consts c, const Params* __restrict__ prm, const T* __restrict__ ipt,
   const T* d = (comp == 0 ? d0 : comp == 1 ? d1 : d2) + (size_t)ioff * P + col;
   T* out = (comp == 0 ? e0 : comp == 1 ? e1 : e2) + (size_t)ioff * P + col;
   const T ob = act ? (comp == 0 ? o0 : comp == 1 ? o1 : o2)[col] : (T)0;
+  // the last segment advances the outflow plane (its old values are no longer read)
+  if (act && k1 == m + 1) (comp == 0 ? u : comp == 1 ? v : w)[(size_t)c.nx * P + col] += ob;
   // inflow-face increment (u) or twice the inflow-value increment (v, w ghost)
   const T ib = (act && inc) ? (comp == 0 ? (T)1 : (T)2) * inc[(size_t)comp * P + col] : (T)0;
   // every lane copies its column of every plane with cp.async (each warp
@@ -919,7 +1021,8 @@ __global__ void __launch_bounds__(256)
 k_af_xv(Consts c, const Params* __restrict__ prm, const T* __restrict__ ipt,
         const T* __restrict__ d0, const T* __restrict__ d1, const T* __restrict__ d2,
         T* __restrict__ e0, T* __restrict__ e1, T* __restrict__ e2, const T* __restrict__ o0,
-        const T* __restrict__ o1, const T* __restrict__ o2, const T* __restrict__ inc) {
+        const T* __restrict__ o1, const T* __restrict__ o2, const T* __restrict__ inc, T* __restrict__ u, T* __restrict__ v,
+        T* __restrict__ w) {
   const int P = c.ny * c.nz;
   const int col = blockIdx.x * blockDim.x + threadIdx.x;
   const int comp = blockIdx.z;
@@ -935,6 +1038,7 @@ k_af_xv(Consts c, const Params* __restrict__ prm, const T* __restrict__ ipt,
   const T* d = (comp == 0 ? d0 : comp == 1 ? d1 : d2) + (size_t)ioff * P + col;
   T* out = (comp == 0 ? e0 : comp == 1 ? e1 : e2) + (size_t)ioff * P + col;
   const T ob = (comp == 0 ? o0 : comp == 1 ? o1 : o2)[col];
+  if (k1 == m + 1) (comp == 0 ? u : comp == 1 ? v : w)[(size_t)c.nx * P + col] += ob;   // as in k_af_xr
   const T ib = inc ? (comp == 0 ? (T)1 : (T)2) * inc[(size_t)comp * P + col] : (T)0;
   // forward warm-up over ks .. k0-1 (values not kept)
   T y = 0;
@@ -1439,28 +1543,7 @@ k_af_z_pipe(Consts c, Params* __restrict__ prm, const T* __restrict__ taps,
 }
 
 // ---------------------------------------------------------------- mass fix + divergence (A7)
-// Q_in, Q_out over the inflow/outflow faces (FP64, fixed summation order);
-// the shift (Q_in - Q_out) / (Ly Lz) goes onto the outflow face.
-// reduce the outflow kernel's per-block flux partials (fixed order)
-__global__ void k_mass(Consts c, Params* prm, const double* __restrict__ qpart, int nb) {
-  __shared__ double scratch[32];
-  double qi = 0.0, qo = 0.0;
-  for (int b = threadIdx.x; b < nb; b += blockDim.x) {
-    qi += qpart[2 * b];
-    qo += qpart[2 * b + 1];
-  }
-  qi = block_sum(qi, scratch);
-  __syncthreads();
-  qo = block_sum(qo, scratch);
-  if (threadIdx.x == 0) {
-    const double h2 = c.h * c.h;
-    prm->q_in = qi * h2;
-    prm->q_out = qo * h2;
-    prm->mass_shift = (qi - qo) * h2 / (c.ly * c.lz);
-    prm->f_mass_shift = (float)prm->mass_shift;
-  }
-}
-
+// (the mass fix's shift comes from the outflow kernel)
 template <class T>
 __global__ void __launch_bounds__(TK* TJ)
 k_div(Consts c, const Params* __restrict__ prm, T* __restrict__ u, const T* __restrict__ v,
@@ -1842,62 +1925,20 @@ static const T* inflow_cur_w(const Consts& c, const Fields<T>& f) { return inflo
 template <class T>
 static const T* inflow_inc(const Consts& c, const Fields<T>& f) { return inflow_plane(c, f, 5); }
 
-// mean of the pending u plane, FP64, fixed order (one block)
 template <class T>
-__global__ void k_inflow_mean(Consts c, const T* __restrict__ pu, double* __restrict__ mean) {
-  __shared__ double scratch[32];
-  const int P = c.ny * c.nz;
-  double s = 0.0;
-  for (int q = threadIdx.x; q < P; q += blockDim.x) s += (double)pu[q];
-  s = block_sum(s, scratch);
-  if (threadIdx.x == 0) *mean = s / P;
-}
-
-// the new inflow time level: u_in = pending u - mean + U on face 0, the
-// boundary increments for the x factor, and the current v, w planes
-template <class T>
-__global__ void k_inflow_advance(Consts c, T* __restrict__ blk, const double* __restrict__ mean,
-                                 T* __restrict__ u) {
-  const int P = c.ny * c.nz;
-  const int jk = blockIdx.x * blockDim.x + threadIdx.x;
-  if (jk >= P) return;
-  T* pu = blk;
-  T* pv = blk + P;
-  T* pw = blk + 2 * (size_t)P;
-  T* cv = blk + 3 * (size_t)P;
-  T* cw = blk + 4 * (size_t)P;
-  T* iu = blk + 5 * (size_t)P;
-  T* iv = blk + 6 * (size_t)P;
-  T* iw = blk + 7 * (size_t)P;
-  const T un = (T)((double)pu[jk] - *mean + c.u_in);
-  iu[jk] = un - u[jk];
-  u[jk] = un;
-  const T vn = pv[jk], wn = pw[jk];
-  iv[jk] = vn - cv[jk];
-  iw[jk] = wn - cw[jk];
-  cv[jk] = vn;
-  cw[jk] = wn;
-}
-
-template <class T>
-void launch_inflow(const Consts& c, const Fields<T>& f, int cur, cudaStream_t s) {
-  if (!f.inflow) return;
-  const int P = c.ny * c.nz;
-  k_inflow_mean<T><<<1, 1024, 0, s>>>(c, f.inflow, f.inflow_mean);
-  k_inflow_advance<T><<<(P + 255) / 256, 256, 0, s>>>(c, f.inflow, f.inflow_mean, f.u[cur]);
-}
-
-template <class T>
-void launch_begin_step(const Consts& c, const Fields<T>& f, cudaStream_t s) {
+void launch_begin_step(const Consts& c, const Fields<T>& f, cudaStream_t s, bool advance) {
   const double tol = sizeof(T) == 8 ? 1e-17 : 1e-9;
-  k_begin_step<<<1, 1024, 0, s>>>(c, f.prm, f.partial, f.n_partial, tol, hmax_of<T>());
+  k_begin_step<<<1, 1024, 0, s>>>(c, f.prm, f.partial, f.n_partial, std::log(tol), hmax_of<T>(), advance ? 1 : 0);
 }
+void launch_end_step(Params* prm, cudaStream_t s) { k_end_step<<<1, 1, 0, s>>>(prm); }
 
 template <class T>
-void launch_af_tables(const Consts& c, const Fields<T>& f, cudaStream_t s) {
-  const int n = table_entries(c);
-  k_af_tables<<<(n + TAB_THREADS - 1) / TAB_THREADS, TAB_THREADS, 0, s>>>(c, f.prm, f.ipt, f.iptf,
-                                                                          f.taps, f.tapsf);
+void launch_head_side(const Consts& c, const Fields<T>& f, int cur, cudaStream_t s) {
+  const int ntab = (table_entries(c) + OUT_THREADS - 1) / OUT_THREADS;
+  const int rest = f.inflow ? 1 : outflow_blocks(c);
+  k_head_side<T><<<ntab + rest, OUT_THREADS, 0, s>>>(c, f.prm, f.ipt, f.iptf, f.taps, f.tapsf, ntab, f.u[cur], f.v[cur],
+                                                     f.w[cur], f.dout[0], f.dout[1], f.dout[2], f.qpart, f.ticket,
+                                                     (const T*)f.inflow, f.inflow_mean);
 }
 
 template <class T>
@@ -2000,10 +2041,12 @@ void launch_rhs_cases(const RhsCase<T>* table, int ncases, int total, int blocks
   k_rhs_cases<T><<<blocks, dim3(TK, TJ), 0, s>>>(table, ncases, total);
 }
 
+// the outflow and mass fix in a launch of their own: after the explicit stage
+// with a prescribed inflow (launch_head_side has taken the mean)
 template <class T>
 void launch_outflow(const Consts& c, const Fields<T>& f, int cur, cudaStream_t s) {
-  k_outflow<T><<<outflow_blocks(c), OUT_THREADS, 0, s>>>(c, f.prm, f.u[cur], f.v[cur], f.w[cur],
-                                                         f.dout[0], f.dout[1], f.dout[2], f.qpart);
+  k_outflow<T><<<outflow_blocks(c), OUT_THREADS, 0, s>>>(c, f.prm, f.u[cur], f.v[cur], f.w[cur], f.dout[0], f.dout[1],
+                                                         f.dout[2], f.qpart, f.ticket, f.inflow, f.inflow_mean);
 }
 
 template <class T>
@@ -2019,24 +2062,23 @@ void launch_af_x(const Consts& c, const Fields<T>& f, int cur, cudaStream_t s) {
       if (xv == 16)
         k_af_xv<T, 16><<<grid, 256, 0, s>>>(c, f.prm, tab, f.d[0], f.d[1], f.d[2], f.e[0], f.e[1],
                                             f.e[2], f.dout[0], f.dout[1], f.dout[2],
-                                            inflow_inc(c, f));
+                                            inflow_inc(c, f), f.u[cur], f.v[cur], f.w[cur]);
       else
         k_af_xv<T, 24><<<grid, 256, 0, s>>>(c, f.prm, tab, f.d[0], f.d[1], f.d[2], f.e[0], f.e[1],
                                             f.e[2], f.dout[0], f.dout[1], f.dout[2],
-                                            inflow_inc(c, f));
+                                            inflow_inc(c, f), f.u[cur], f.v[cur], f.w[cur]);
       return;
     }
     // otherwise segments of 32 or 64 planes staged in shared memory by warps
     if (c.afx_planes <= 40) {
       k_af_xr<T, 32><<<dim3((P + 31) / 32, (c.nx + 31) / 32, 3), 32, 0, s>>>(
           c, f.prm, tab, f.d[0], f.d[1], f.d[2], f.e[0], f.e[1], f.e[2], f.dout[0], f.dout[1],
-          f.dout[2], inflow_inc(c, f));
+          f.dout[2], inflow_inc(c, f), f.u[cur], f.v[cur], f.w[cur]);
     } else {
       k_af_xr<T, 64><<<dim3((P + 31) / 32, (c.nx + 63) / 64, 3), 32, 0, s>>>(
           c, f.prm, tab, f.d[0], f.d[1], f.d[2], f.e[0], f.e[1], f.e[2], f.dout[0], f.dout[1],
-          f.dout[2], inflow_inc(c, f));
+          f.dout[2], inflow_inc(c, f), f.u[cur], f.v[cur], f.w[cur]);
     }
-    (void)cur;
   }
 }
 
@@ -2104,12 +2146,6 @@ void launch_af(const Consts& c, const Fields<T>& f, int cur, cudaStream_t s) {
 }
 
 template <class T>
-void launch_mass(const Consts& c, const Fields<T>& f, int cur, cudaStream_t s) {
-  k_mass<<<1, 1024, 0, s>>>(c, f.prm, f.qpart, outflow_blocks(c));
-  (void)cur;
-}
-
-template <class T>
 void launch_div(const Consts& c, const Fields<T>& f, int cur, bool initial, cudaStream_t s) {
   if (const RunShape r = run_shape<T>(c, c.nx, 4); r.rows) {
     k_div_vec<T><<<dim3(c.ny / r.rows, (c.nx + r.xch - 1) / r.xch), r.threads, 0, s>>>(
@@ -2120,16 +2156,10 @@ void launch_div(const Consts& c, const Fields<T>& f, int cur, bool initial, cuda
                                                     initial ? 1 : 0);
 }
 
-template <class T>
-void launch_mass_div(const Consts& c, const Fields<T>& f, int cur, bool initial, cudaStream_t s) {
-  if (!initial) launch_mass(c, f, cur, s);
-  launch_div(c, f, cur, initial, s);
-}
-
 // phi = phi_a + phi_b when phi_b is given (the mixed solve's predictor and
 // correction), phi_a = f.phi when not given
 template <class T>
-void launch_project_only(const Consts& c, const Fields<T>& f, int cur, bool initial, cudaStream_t s,
+void launch_project(const Consts& c, const Fields<T>& f, int cur, bool initial, cudaStream_t s,
                          const T* phi_a, const T* phi_b, const void* phi_b16) {
   if (!phi_a) phi_a = f.phi;
   if (const RunShape r = run_shape<T>(c, c.nx + 1, 8); r.rows) {
@@ -2159,13 +2189,6 @@ void launch_project_only(const Consts& c, const Fields<T>& f, int cur, bool init
 }
 
 template <class T>
-void launch_project(const Consts& c, const Fields<T>& f, int cur, bool initial, cudaStream_t s,
-                    const T* phi_a, const T* phi_b, const void* phi_b16) {
-  launch_project_only(c, f, cur, initial, s, phi_a, phi_b, phi_b16);
-  if (!initial) k_end_step<<<1, 1, 0, s>>>(f.prm);
-}
-
-template <class T>
 void launch_stats(const Consts& c, const Fields<T>& f, int cur, double* out, cudaStream_t s) {
   k_stats<T><<<grid3(c, c.nx + 1), dim3(TK, TJ), 0, s>>>(c, f.u[cur], f.v[cur], f.w[cur], out);
 }
@@ -2192,23 +2215,18 @@ template int partial_count<float>(const Consts&);
 template int partial_count<double>(const Consts&);
 
 #define INST(T)                                                                                \
-  template void launch_begin_step<T>(const Consts&, const Fields<T>&, cudaStream_t);           \
+  template void launch_begin_step<T>(const Consts&, const Fields<T>&, cudaStream_t, bool);     \
+  template void launch_head_side<T>(const Consts&, const Fields<T>&, int, cudaStream_t);        \
   template void launch_rhs<T>(const Consts&, const Fields<T>&, int, cudaStream_t);             \
   template RhsCase<T> rhs_case<T>(const Consts&, const Fields<T>&, int);                       \
   template void launch_rhs_cases<T>(const RhsCase<T>*, int, int, int, cudaStream_t);          \
-  template void launch_af_tables<T>(const Consts&, const Fields<T>&, cudaStream_t);             \
-  template void launch_inflow<T>(const Consts&, const Fields<T>&, int, cudaStream_t);           \
   template void launch_outflow<T>(const Consts&, const Fields<T>&, int, cudaStream_t);         \
   template void launch_af<T>(const Consts&, const Fields<T>&, int, cudaStream_t);              \
   template void launch_af_x<T>(const Consts&, const Fields<T>&, int, cudaStream_t);            \
   template void launch_af_y<T>(const Consts&, const Fields<T>&, int, cudaStream_t);            \
   template void launch_af_z<T>(const Consts&, const Fields<T>&, int, cudaStream_t);            \
   template bool launch_af_yz<T>(const Consts&, const Fields<T>&, int, cudaStream_t);           \
-  template void launch_mass<T>(const Consts&, const Fields<T>&, int, cudaStream_t);            \
   template void launch_div<T>(const Consts&, const Fields<T>&, int, bool, cudaStream_t);       \
-  template void launch_project_only<T>(const Consts&, const Fields<T>&, int, bool, cudaStream_t, const T*, \
-                                       const T*, const void*);                                     \
-  template void launch_mass_div<T>(const Consts&, const Fields<T>&, int, bool, cudaStream_t);  \
   template void launch_project<T>(const Consts&, const Fields<T>&, int, bool, cudaStream_t, const T*, \
                                   const T*, const void*);                                          \
   template void launch_stats<T>(const Consts&, const Fields<T>&, int, double*, cudaStream_t);

@@ -26,7 +26,7 @@ struct Fields {
   T* tw_y; T* tw_z;           // FFT twiddles exp(-2 pi i t / N), t < N/2 (re, im)
   double* partial;            // per-block partial maxima of the CFL speed
   double* qpart;              // per-block inflow/outflow flux partials
-  double* mean00;             // line mean of the Poisson mode (0, 0)
+  int* ticket;                // blocks of the outflow kernel that have finished (0 between launches)
   // prescribed inflow (null when disabled): 8 planes of ny * nz values:
   // pending u, v, w (next time level, written by the caller), current v, w
   // (ghosts of the explicit stage), increments u, v, w (x factor's first row)
@@ -124,10 +124,14 @@ struct SlabDev {
 };
 
 // ---- fluid.cu
-template <class T> void launch_begin_step(const Consts& c, const Fields<T>& f, cudaStream_t s);
+// advance: the previous step of the same call ends here (its clock)
+template <class T> void launch_begin_step(const Consts& c, const Fields<T>& f, cudaStream_t s, bool advance);
+void launch_end_step(Params* prm, cudaStream_t s);
 template <class T> void launch_speed_check(const Consts& c, const Fields<T>& f, cudaStream_t s);
-template <class T> void launch_af_tables(const Consts& c, const Fields<T>& f, cudaStream_t s);
-template <class T> void launch_inflow(const Consts& c, const Fields<T>& f, int cur, cudaStream_t s);
+// beside the explicit stage: the implicit factors' tables and the outflow's
+// increments with the mass fix, or the mean of the pending inflow, which
+// launch_outflow then needs after the explicit stage
+template <class T> void launch_head_side(const Consts& c, const Fields<T>& f, int cur, cudaStream_t s);
 template <class T> void launch_rhs(const Consts& c, const Fields<T>& f, int cur, cudaStream_t s);
 template <class T> RhsCase<T> rhs_case(const Consts& c, const Fields<T>& f, int cur);
 // the explicit stage of every case of `table` (device memory, ncases
@@ -145,13 +149,8 @@ template <class T> bool launch_dht2d(const Consts& c, const Fields<T>& f, cudaSt
 bool dht2d_plane_supported(int ny, int nz);
 bool launch_dht2d_on(const Consts& c, const Fields<float>& f, const float* in, float* out, cudaStream_t s);
 bool dht2d_planes_fp32(const float* in, float* out, int nplanes, const float* tw, cudaStream_t s);
-template <class T> void launch_mass(const Consts& c, const Fields<T>& f, int cur, cudaStream_t s);
 template <class T> void launch_div(const Consts& c, const Fields<T>& f, int cur, bool initial, cudaStream_t s);
 // phi = phi_a (f.phi when null) + phi_b (FP32) or + phi_b16 (bfloat16, FP32 fields only)
-template <class T> void launch_project_only(const Consts& c, const Fields<T>& f, int cur, bool initial, cudaStream_t s,
-                                            const T* phi_a = nullptr, const T* phi_b = nullptr,
-                                            const void* phi_b16 = nullptr);
-template <class T> void launch_mass_div(const Consts& c, const Fields<T>& f, int cur, bool initial, cudaStream_t s);
 template <class T> void launch_project(const Consts& c, const Fields<T>& f, int cur, bool initial, cudaStream_t s,
                                        const T* phi_a = nullptr, const T* phi_b = nullptr,
                                        const void* phi_b16 = nullptr);
