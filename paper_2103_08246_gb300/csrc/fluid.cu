@@ -542,13 +542,22 @@ k_rhs_pipe(Consts c, Params* __restrict__ prm, const T* __restrict__ u,
 // The ring stages u, v, w (rows j0-1 .. j0+TJ) and p (rows j0-1 .. j0+TJ-1)
 // of one x plane per slot; N^{n-1} is read straight from global memory into
 // registers (it has no neighbours in the stencil). A block is TJ rows of
-// runs (256 threads at nz = 256); FP32 fits two blocks per SM.
+// runs (256 threads at nz = 256), two blocks per SM. FP64 is bound by its pipe:
+// with the fluxes shared (86 -> about 75 instructions per cell) and a second
+// block per SM 512 x 256 x 256 takes 4.94 instead of 5.88 ms. (FP32, bound by
+// memory, is slower that way, 0.320 against 0.298 ms: registers and a longer
+// chain from plane to plane.)
 template <class T>
 struct RhsVec {
   static constexpr int E = 16 / sizeof(T);
   static constexpr int TJ = sizeof(T) == 4 ? 4 : 2;
   static constexpr int RW = TJ + 2;
-  static constexpr int ROWS = 3 * RW + TJ + 1;
+  // FP32 stages p as well; FP64 reads it straight from global memory, which
+  // brings the ring at nz = 256 from 123 to 98 KB and a second block onto the SM
+  static constexpr bool PS = sizeof(T) == 4;
+  // FP64, bound by its pipe: every flux once where a thread holds both sides
+  static constexpr bool SHARE = sizeof(T) == 8;
+  static constexpr int ROWS = 3 * RW + (PS ? TJ + 1 : 0);
   static constexpr int STAGES = 4;
 };
 template <class T>
@@ -612,7 +621,7 @@ k_rhs_vec(Consts c, Params* __restrict__ prm, const T* __restrict__ u, const T* 
     const bool has_p = (q >= 0 && q <= nx - 1);
     const int slot = t % NS;
     T* st = stage_ptr(slot);
-    const uint32_t bytes = (uint32_t)((3 * RW + (has_p ? TJ + 1 : 0)) * rowb);
+    const uint32_t bytes = (uint32_t)((3 * RW + (has_p && RV::PS ? TJ + 1 : 0)) * rowb);
     mbar_arrive_expect_tx(&full[slot], bytes);
     for (int r = 0; r < RW; ++r) {
       int jj = j0 - 1 + r;
@@ -622,7 +631,7 @@ k_rhs_vec(Consts c, Params* __restrict__ prm, const T* __restrict__ u, const T* 
       bulk_g2s(st + (size_t)(RW + r) * nz, v + g, (uint32_t)rowb, &full[slot]);
       bulk_g2s(st + (size_t)(2 * RW + r) * nz, w + g, (uint32_t)rowb, &full[slot]);
     }
-    if (has_p)
+    if (has_p && RV::PS)
       for (int r = 0; r < TJ + 1; ++r) {
         int jj = j0 - 1 + r;
         jj = jj < 0 ? jj + ny : jj;
@@ -667,6 +676,11 @@ k_rhs_vec(Consts c, Params* __restrict__ prm, const T* __restrict__ u, const T* 
     if (lane == 31 || k0 + E >= nz) v = row[kpE];
     return v;
   };
+  // carried along x: the x fluxes of u, v, w at the planes' lower side, and p
+  T Fuu[E], Fuv[E], Fuw[E], pa[E];
+#pragma unroll
+  for (int e = 0; e < E; ++e) Fuu[e] = Fuv[e] = Fuw[e] = pa[e] = (T)0;
+  const size_t P = plane(c);
   for (int i = ib; i < ie; ++i) {
     const int ta = i - ib, tb = ta + 1, tc = ta + 2;
     const size_t id = ((size_t)i * ny + j) * nz + k0;
@@ -695,7 +709,6 @@ k_rhs_vec(Consts c, Params* __restrict__ prm, const T* __restrict__ u, const T* 
     const T* Wa = A + 2 * RW * nz;
     const T* Wb = B + 2 * RW * nz;
     const T* Wc = C + 2 * RW * nz;
-    const T* Pa = A + 3 * RW * nz;
     const T* Pb = B + 3 * RW * nz;
     const T sgn = i - 1 < 0 ? (T)-1 : (T)1;   // inflow ghost of v, w: 2 q_in - q_0
     T gv[E], gw[E];
@@ -731,80 +744,173 @@ k_rhs_vec(Consts c, Params* __restrict__ prm, const T* __restrict__ u, const T* 
     lds_run<T, E>(Wb + Rp + k0, wbp);
     lds_run<T, E>(Wa + R + k0, wa);
     lds_run<T, E>(Wc + R + k0, wc);
-    lds_run<T, E>(Pb + R + k0, pb);
-    lds_run<T, E>(Pb + Rm + k0, pbm);
+    T pb_l;
+    if constexpr (RV::PS) {
+      lds_run<T, E>(Pb + R + k0, pb);
+      lds_run<T, E>(Pb + Rm + k0, pbm);
+      pb_l = left(pb[E - 1], Pb + R);
+    } else {
+      const T* prow = p + (size_t)i * P + (size_t)j * nz;
+      ldg_run<T, E>(prow + k0, pb);
+      ldg_run<T, E>(p + (size_t)i * P + (size_t)(j == 0 ? ny - 1 : j - 1) * nz + k0, pbm);
+      pb_l = left(pb[E - 1], prow);
+    }
     const T ub_l = left(ub[E - 1], Ub + R), ub_r = right(ub[0], Ub + R);
     const T uc_l = left(uc[E - 1], Uc + R);
     const T vb_l = left(vb[E - 1], Vb + R), vb_r = right(vb[0], Vb + R);
     const T vbp_l = left(vbp[E - 1], Vb + Rp);
     const T wb_l = left(wb[E - 1], Wb + R), wb_r = right(wb[0], Wb + R);
     const T wa_r = right(wa[0], Wa + R), wbm_r = right(wbm[0], Wb + Rm);
-    const T pb_l = left(pb[E - 1], Pb + R);
     T No[E], Do[E];
-    // Flux differences with the halves folded into qh = ih / 4:
-    // (a+b)/2 (c+d)/2 products become (a+b)(c+d), and each face pair is one
-    // product and one fused multiply-add. RHS = -dt alpha N - dt beta N^{n-1}
-    // + dt nu ih^2 Lraw - dt ih (p_c - p_w), every term one FMA.
-    // u on face i (interior faces only; no inflow ghost enters it)
-    if (i >= 1) {
-      T ua[E], pa[E];
+    if constexpr (RV::SHARE) {
+      // Each flux is computed once where the thread holds both sides: the x
+      // fluxes carry over from the last plane (and are the lower y and z fluxes of
+      // u), the yz flux serves v and w, z faces inside the run serve both cells.
+      T ua[E];
       lds_run<T, E>(Ua + R + k0, ua);
-      lds_run<T, E>(Pa + R + k0, pa);
+      if (i == ib) {
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+          const T s = ua[e] + ub[e];
+          Fuu[e] = s * s;
+          Fuv[e] = (ubm[e] + ub[e]) * (sgn * va[e] + gv[e] + vb[e]);
+          Fuw[e] = ((e == 0 ? ub_l : ub[e - 1]) + ub[e]) * (sgn * wa[e] + gw[e] + wb[e]);
+        }
+        if (i >= 1) ldg_run<T, E>(p + (size_t)(i - 1) * P + (size_t)j * nz + k0, pa);
+      }
+      // u on face i (interior faces only; no inflow ghost enters it)
+      const T fuw_r = (ub[E - 1] + ub_r) * (wa_r + wb_r);   // the run's upper z face
 #pragma unroll
       for (int e = 0; e < E; ++e) {
-        const T c0 = ub[e];
+        const T c0 = ub[e], sp = c0 + uc[e], fn = sp * sp;
         const T uzp = e == E - 1 ? ub_r : ub[e + 1], uzm = e == 0 ? ub_l : ub[e - 1];
-        const T wap = e == E - 1 ? wa_r : wa[e + 1], wbp1 = e == E - 1 ? wb_r : wb[e + 1];
-        const T sp = c0 + uc[e], sm = ua[e] + c0;
-        const T fx = sp * sp - sm * sm;
-        const T fy = (c0 + ubp[e]) * (vap[e] + vbp[e]) - (ubm[e] + c0) * (va[e] + vb[e]);
-        const T fz = (c0 + uzp) * (wap + wbp1) - (uzm + c0) * (wa[e] + wb[e]);
-        const T N = qh * (fx + fy + fz);
+        const T fy = (c0 + ubp[e]) * (vap[e] + vbp[e]) - Fuv[e];
+        const T fz = (e == E - 1 ? fuw_r : Fuw[e + 1]) - Fuw[e];
+        const T N = qh * ((fn - Fuu[e]) + fy + fz);
         const T L = uc[e] + ua[e] + ubp[e] + ubm[e] + uzp + uzm - (T)6 * c0;
         No[e] = N;
         Do[e] = mda * N + (mdb * Np0[e] + (cdn * L - cdg * (pb[e] - pa[e])));
+        Fuu[e] = fn;
       }
-      stg_run<T, E>(n0 + id, No);
-      stg_run<T, E>(d0 + id, Do);
-    }
-    // v at (i + 1/2, j, k + 1/2)
+      if (i >= 1) {
+        stg_run<T, E>(n0 + id, No);
+        stg_run<T, E>(d0 + id, Do);
+      }
+      // the yz fluxes of the run's E + 1 z faces at y face j
+      T G[E + 1];
 #pragma unroll
-    for (int e = 0; e < E; ++e) {
-      const T c0 = vb[e];
-      const T vxp = vc[e], vxm = sgn * va[e] + gv[e];
-      const T vzp = e == E - 1 ? vb_r : vb[e + 1], vzm = e == 0 ? vb_l : vb[e - 1];
-      const T wbp1 = e == E - 1 ? wb_r : wb[e + 1], wbmp1 = e == E - 1 ? wbm_r : wbm[e + 1];
-      const T fx = (ucm[e] + uc[e]) * (c0 + vxp) - (ubm[e] + ub[e]) * (vxm + c0);
-      const T sp = c0 + vbp[e], sm = vbm[e] + c0;
-      const T fy = sp * sp - sm * sm;
-      const T fz = (c0 + vzp) * (wbmp1 + wbp1) - (vzm + c0) * (wbm[e] + wb[e]);
-      const T N = qh * (fx + fy + fz);
-      const T L = vxp + vxm + vbp[e] + vbm[e] + vzp + vzm - (T)6 * c0;
-      No[e] = N;
-      Do[e] = mda * N + (mdb * Np1[e] + (cdn * L - cdg * (pb[e] - pbm[e])));
-    }
-    stg_run<T, E>(n1 + id, No);
-    stg_run<T, E>(d1 + id, Do);
-    // w at (i + 1/2, j + 1/2, k)
+      for (int e = 0; e <= E; ++e) {
+        const T vl = e == 0 ? vb_l : vb[e == 0 ? 0 : e - 1], vr = e == E ? vb_r : vb[e == E ? 0 : e];
+        const T wl = e == E ? wbm_r : wbm[e == E ? 0 : e], wr = e == E ? wb_r : wb[e == E ? 0 : e];
+        G[e] = (vl + vr) * (wl + wr);
+      }
+      // v at (i + 1/2, j, k + 1/2)
 #pragma unroll
-    for (int e = 0; e < E; ++e) {
-      const T c0 = wb[e];
-      const T wxp = wc[e], wxm = sgn * wa[e] + gw[e];
-      const T wzp = e == E - 1 ? wb_r : wb[e + 1], wzm = e == 0 ? wb_l : wb[e - 1];
-      const T ucl = e == 0 ? uc_l : uc[e - 1], ubl = e == 0 ? ub_l : ub[e - 1];
-      const T vbpl = e == 0 ? vbp_l : vbp[e - 1], vbl = e == 0 ? vb_l : vb[e - 1];
-      const T pbl = e == 0 ? pb_l : pb[e - 1];
-      const T fx = (ucl + uc[e]) * (c0 + wxp) - (ubl + ub[e]) * (wxm + c0);
-      const T fy = (vbpl + vbp[e]) * (c0 + wbp[e]) - (vbl + vb[e]) * (wbm[e] + c0);
-      const T sp = c0 + wzp, sm = wzm + c0;
-      const T fz = sp * sp - sm * sm;
-      const T N = qh * (fx + fy + fz);
-      const T L = wxp + wxm + wbp[e] + wbm[e] + wzp + wzm - (T)6 * c0;
-      No[e] = N;
-      Do[e] = mda * N + (mdb * Np2[e] + (cdn * L - cdg * (pb[e] - pbl)));
+      for (int e = 0; e < E; ++e) {
+        const T c0 = vb[e];
+        const T vxp = vc[e], vxm = sgn * va[e] + gv[e];
+        const T vzp = e == E - 1 ? vb_r : vb[e + 1], vzm = e == 0 ? vb_l : vb[e - 1];
+        const T fn = (ucm[e] + uc[e]) * (c0 + vxp);
+        const T sp = c0 + vbp[e], sm = vbm[e] + c0;
+        const T fy = sp * sp - sm * sm;
+        const T N = qh * ((fn - Fuv[e]) + fy + (G[e + 1] - G[e]));
+        const T L = vxp + vxm + vbp[e] + vbm[e] + vzp + vzm - (T)6 * c0;
+        No[e] = N;
+        Do[e] = mda * N + (mdb * Np1[e] + (cdn * L - cdg * (pb[e] - pbm[e])));
+        Fuv[e] = fn;
+      }
+      stg_run<T, E>(n1 + id, No);
+      stg_run<T, E>(d1 + id, Do);
+      // w at (i + 1/2, j + 1/2, k)
+      T fz = (wb_l + wb[0]) * (wb_l + wb[0]);   // the lower z face, then the upper one of each cell
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        const T c0 = wb[e];
+        const T wxp = wc[e], wxm = sgn * wa[e] + gw[e];
+        const T wzp = e == E - 1 ? wb_r : wb[e + 1], wzm = e == 0 ? wb_l : wb[e - 1];
+        const T ucl = e == 0 ? uc_l : uc[e - 1];
+        const T vbpl = e == 0 ? vbp_l : vbp[e - 1];
+        const T pbl = e == 0 ? pb_l : pb[e - 1];
+        const T fn = (ucl + uc[e]) * (c0 + wxp);
+        const T fy = (vbpl + vbp[e]) * (c0 + wbp[e]) - G[e];
+        const T sp = c0 + wzp, fzn = sp * sp;
+        const T N = qh * ((fn - Fuw[e]) + fy + (fzn - fz));
+        const T L = wxp + wxm + wbp[e] + wbm[e] + wzp + wzm - (T)6 * c0;
+        No[e] = N;
+        Do[e] = mda * N + (mdb * Np2[e] + (cdn * L - cdg * (pb[e] - pbl)));
+        Fuw[e] = fn;
+        fz = fzn;
+      }
+      stg_run<T, E>(n2 + id, No);
+      stg_run<T, E>(d2 + id, Do);
+#pragma unroll
+      for (int e = 0; e < E; ++e) pa[e] = pb[e];
+    } else {
+      // Flux differences with the halves folded into qh = ih / 4:
+      // (a+b)/2 (c+d)/2 products become (a+b)(c+d), and each face pair is one
+      // product and one fused multiply-add. RHS = -dt alpha N - dt beta N^{n-1}
+      // + dt nu ih^2 Lraw - dt ih (p_c - p_w), every term one FMA.
+      // u on face i (interior faces only; no inflow ghost enters it)
+      if (i >= 1) {
+        T ua[E];
+        lds_run<T, E>(Ua + R + k0, ua);
+        lds_run<T, E>(A + 3 * RW * nz + R + k0, pa);
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+          const T c0 = ub[e];
+          const T uzp = e == E - 1 ? ub_r : ub[e + 1], uzm = e == 0 ? ub_l : ub[e - 1];
+          const T wap = e == E - 1 ? wa_r : wa[e + 1], wbp1 = e == E - 1 ? wb_r : wb[e + 1];
+          const T sp = c0 + uc[e], sm = ua[e] + c0;
+          const T fx = sp * sp - sm * sm;
+          const T fy = (c0 + ubp[e]) * (vap[e] + vbp[e]) - (ubm[e] + c0) * (va[e] + vb[e]);
+          const T fz = (c0 + uzp) * (wap + wbp1) - (uzm + c0) * (wa[e] + wb[e]);
+          const T N = qh * (fx + fy + fz);
+          const T L = uc[e] + ua[e] + ubp[e] + ubm[e] + uzp + uzm - (T)6 * c0;
+          No[e] = N;
+          Do[e] = mda * N + (mdb * Np0[e] + (cdn * L - cdg * (pb[e] - pa[e])));
+        }
+        stg_run<T, E>(n0 + id, No);
+        stg_run<T, E>(d0 + id, Do);
+      }
+      // v at (i + 1/2, j, k + 1/2)
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        const T c0 = vb[e];
+        const T vxp = vc[e], vxm = sgn * va[e] + gv[e];
+        const T vzp = e == E - 1 ? vb_r : vb[e + 1], vzm = e == 0 ? vb_l : vb[e - 1];
+        const T wbp1 = e == E - 1 ? wb_r : wb[e + 1], wbmp1 = e == E - 1 ? wbm_r : wbm[e + 1];
+        const T fx = (ucm[e] + uc[e]) * (c0 + vxp) - (ubm[e] + ub[e]) * (vxm + c0);
+        const T sp = c0 + vbp[e], sm = vbm[e] + c0;
+        const T fy = sp * sp - sm * sm;
+        const T fz = (c0 + vzp) * (wbmp1 + wbp1) - (vzm + c0) * (wbm[e] + wb[e]);
+        const T N = qh * (fx + fy + fz);
+        const T L = vxp + vxm + vbp[e] + vbm[e] + vzp + vzm - (T)6 * c0;
+        No[e] = N;
+        Do[e] = mda * N + (mdb * Np1[e] + (cdn * L - cdg * (pb[e] - pbm[e])));
+      }
+      stg_run<T, E>(n1 + id, No);
+      stg_run<T, E>(d1 + id, Do);
+      // w at (i + 1/2, j + 1/2, k)
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        const T c0 = wb[e];
+        const T wxp = wc[e], wxm = sgn * wa[e] + gw[e];
+        const T wzp = e == E - 1 ? wb_r : wb[e + 1], wzm = e == 0 ? wb_l : wb[e - 1];
+        const T ucl = e == 0 ? uc_l : uc[e - 1], ubl = e == 0 ? ub_l : ub[e - 1];
+        const T vbpl = e == 0 ? vbp_l : vbp[e - 1], vbl = e == 0 ? vb_l : vb[e - 1];
+        const T pbl = e == 0 ? pb_l : pb[e - 1];
+        const T fx = (ucl + uc[e]) * (c0 + wxp) - (ubl + ub[e]) * (wxm + c0);
+        const T fy = (vbpl + vbp[e]) * (c0 + wbp[e]) - (vbl + vb[e]) * (wbm[e] + c0);
+        const T sp = c0 + wzp, sm = wzm + c0;
+        const T fz = sp * sp - sm * sm;
+        const T N = qh * (fx + fy + fz);
+        const T L = wxp + wxm + wbp[e] + wbm[e] + wzp + wzm - (T)6 * c0;
+        No[e] = N;
+        Do[e] = mda * N + (mdb * Np2[e] + (cdn * L - cdg * (pb[e] - pbl)));
+      }
+      stg_run<T, E>(n2 + id, No);
+      stg_run<T, E>(d2 + id, Do);
     }
-    stg_run<T, E>(n2 + id, No);
-    stg_run<T, E>(d2 + id, Do);
     __syncthreads();
     // the slot of plane i-1 is free: refill it with the stage NS ahead
     if (tid == 0 && ta + NS < nstage) issue(ta + NS);
