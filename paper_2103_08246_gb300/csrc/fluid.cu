@@ -174,7 +174,7 @@ template void launch_speed_check<double>(const Consts&, const Fields<double>&, c
 //     t_m = (1/r) rho / (1 - rho^2) (rho^m + rho^{n-m}) / (1 - rho^n)
 // Powers by repeated squaring; rho stays below 1/2 within the factors' range
 // (r up to 0.3 in FP64, 1.3 in FP32), so 1 - rho^k does not cancel.
-int table_entries(const Consts& c) { return c.nx + (HMAX + 1) + c.ny + c.nz; }
+int table_entries(const Consts& c) { return 40 + c.nx + (HMAX + 1) + c.ny + c.nz; }   // 40: YZ_TAB below
 
 __device__ inline double int_power(double b, int n) {
   double v = 1.0;
@@ -185,9 +185,27 @@ __device__ inline double int_power(double b, int n) {
   return v;
 }
 
+// after the taps: what every warp of the fused y-z factors and of the divergence
+// needs, rho^(E l) of the 32 lanes (E = nz / 32 points per lane), then
+// 1 / (1 - rho^2), 1 / (1 - rho^nz), rho / r and 1 / (h dt). Computed per thread
+// these took a third of the y-z factors' FP64 instructions.
+constexpr int YZ_TAB = 40;
+__host__ __device__ inline int yz_table(const Consts& c) { return c.ny + c.nz + 32; }
+enum { YZ_INV_R2 = 32, YZ_INV_RN, YZ_RHO_R, YZ_DIV };
+
 __device__ inline void af_table_entry(const Consts& c, const Params* prm, double* ipt, float* iptf, double* taps,
                                       float* tapsf, int q) {
   const double r = prm->r, rho = prm->af_rho;
+  if (q < YZ_TAB) {
+    const double v = q < 32 ? int_power(rho, (c.nz / 32) * q)
+                            : q == YZ_INV_R2 ? 1.0 / (1.0 - rho * rho)
+                                             : q == YZ_INV_RN ? 1.0 / (1.0 - int_power(rho, c.nz))
+                                                              : q == YZ_RHO_R ? rho / r : c.inv_h / prm->dt;
+    taps[yz_table(c) + q] = v;
+    tapsf[yz_table(c) + q] = (float)v;
+    return;
+  }
+  q -= YZ_TAB;
   if (q < c.nx) {
     const int k = q + 1;
     const double odd = int_power(rho, 2 * k - 1);   // rho^(2k-1), and from it 2k, 2k+1, 2k+2
@@ -1334,7 +1352,7 @@ __device__ inline void store_run(T* p, const T (&v)[E]) {
 
 template <class T, int E>
 __global__ void __launch_bounds__(YZ_THREADS)
-k_af_yz(Consts c, const Params* __restrict__ prm, const T* __restrict__ e0,
+k_af_yz(Consts c, const Params* __restrict__ prm, const T* __restrict__ tab, const T* __restrict__ e0,
         const T* __restrict__ e1, const T* __restrict__ e2, T* __restrict__ u,
         T* __restrict__ v, T* __restrict__ w) {
   constexpr int NZ = 32 * E;
@@ -1350,9 +1368,8 @@ k_af_yz(Consts c, const Params* __restrict__ prm, const T* __restrict__ e0,
   // The recursions run on r-scaled values (y' = r y, z' = r z): the 1/r of
   // the forcing moves into one final factor rho / r per output.
   const T rho = pick<T>(prm->af_rho, prm->f_rho);
-  const T rho_ir = rho * pick<T>(1.0 / prm->r, prm->f_ir);
   const int H = prm->af_h;
-  const T inv_1mr2 = (T)1 / ((T)1 - rho * rho);
+  const T inv_1mr2 = tab[YZ_INV_R2];
   // ---- y factor
   for (int k = threadIdx.x; k < NZ; k += YZ_THREADS) {
     const T* col = in + k;
@@ -1381,7 +1398,8 @@ k_af_yz(Consts c, const Params* __restrict__ prm, const T* __restrict__ e0,
 #pragma unroll
       for (int t = 0; t < 8; ++t) buf[t] = (m0 + t < H) ? col[(size_t)((j0 + J + m0 + t) & ymask) * NZ] : (T)0;
 #pragma unroll
-      for (int t = 7; t >= 0; --t) sf = buf[t] + rho * sf;   // zeros beyond H
+      for (int t = 7; t >= 0; --t)
+        if (m0 + t < H) sf = buf[t] + rho * sf;
     }
     T z = (rho * y + sf) * inv_1mr2;
     const int kp = k + (k >> 5);
@@ -1399,18 +1417,8 @@ k_af_yz(Consts c, const Params* __restrict__ prm, const T* __restrict__ e0,
 #pragma unroll
   for (int t = 1; t < E; ++t) rp[t] = rp[t - 1] * rho;
   const T pE = rp[E - 1];                    // rho^E
-  T pl = 1, pr = 1;                          // rho^(E lane), rho^(E (31 - lane))
-  {
-    T b = pE;
-#pragma unroll
-    for (int bit = 0; bit < 5; ++bit) {
-      if ((lane >> bit) & 1) pl *= b;
-      if (((31 - lane) >> bit) & 1) pr *= b;
-      b *= b;
-    }
-  }
-  const T rn = pl * pr * pE;                 // rho^nz
-  const T inv_1mrn = (T)1 / ((T)1 - rn);
+  const T pl = tab[lane], pr = tab[31 - lane];   // rho^(E lane), rho^(E (31 - lane))
+  const T inv_1mrn = tab[YZ_INV_RN];
   // scan steps until the factor rho^(E 2^s) falls below the tolerance of the
   // warm-up length (usually one or two of five)
   T ps[5];
@@ -1424,7 +1432,7 @@ k_af_yz(Consts c, const Params* __restrict__ prm, const T* __restrict__ e0,
       b *= b;
     }
   }
-  const T scale = rho_ir * rho_ir;           // of both factors
+  const T scale = tab[YZ_RHO_R] * tab[YZ_RHO_R];   // of both factors
   for (int r = warp; r < J; r += YZ_THREADS / 32) {
     T* qrow = q + (size_t)(j0 + r) * NZ + lane * E;
     T un[E];
@@ -1813,7 +1821,7 @@ RunShape run_shape(const Consts& c, int planes, int most) {
 
 template <class T>
 __global__ void __launch_bounds__(256)
-k_div_vec(Consts c, const Params* __restrict__ prm, T* __restrict__ u, const T* __restrict__ v,
+k_div_vec(Consts c, const Params* __restrict__ prm, const T* __restrict__ tab, T* __restrict__ u, const T* __restrict__ v,
           const T* __restrict__ w, T* __restrict__ phi, int initial, int xch) {
   constexpr int E = RunTile<T>::E;
   const int nx = c.nx, ny = c.ny, nz = c.nz;
@@ -1824,7 +1832,7 @@ k_div_vec(Consts c, const Params* __restrict__ prm, T* __restrict__ u, const T* 
   const int jp = (j + 1) & (ny - 1), kpE = (k0 + E) & (nz - 1);
   const size_t P = plane(c);
   const T shift = initial ? (T)0 : pick<T>(prm->mass_shift, prm->f_mass_shift);
-  const T sc = initial ? pick<T>(c.inv_h, c.f_inv_h) : pick<T>(c.inv_h / prm->dt, prm->f_sc_div);
+  const T sc = initial ? pick<T>(c.inv_h, c.f_inv_h) : tab[YZ_DIV];
   const int i0 = blockIdx.y * xch, i1 = min(i0 + xch, nx);
   if (i0 >= i1) return;
   T uw[E];
@@ -2190,19 +2198,26 @@ static size_t rhs_stage_bytes(const Consts& c, int tjr) {
 // planes for every grid left a last wave nearly empty or most SMs idle:
 // 512 x 256 x 256 FP32 0.308 -> 0.297 ms (27 planes, exactly four waves),
 // 384 x 256 x 256 0.259 -> 0.228, 64 x 32 x 32 FP64 0.110 -> 0.019 (2 planes).
-// Blocks of fewer planes read more halo: that costs FP64 little (its pipe
-// bounds the stage), and a small FP32 grid nothing, but larger FP32 grids that
-// share the chip in an ensemble 1.5%, so those keep at least 16 planes.
+// Blocks of fewer planes read more halo, which costs a small FP32 grid nothing,
+// but larger FP32 grids that share the chip in an ensemble 1.5%, so those keep
+// at least 16 planes. FP64 is bound by its pipe: the time is that of the SM with
+// the most blocks, planes x blocks, unless its warps are fewer than the five or
+// so that keep the pipe busy (96 x 64 x 128: 0.146 -> 0.127 ms, 7 planes, three
+// blocks per SM, where whole waves of four per SM left some SMs with three). The
+// half block more allows for what else runs beside the stage: one exact round of
+// large blocks lost a third when an SM got one more than its share.
 template <class T>
-static int rhs_wave_planes(const Consts& c, int yblocks, int per_sm) {
+static int rhs_wave_planes(const Consts& c, int yblocks, int per_sm, int warps) {
   const int nx = c.nx;
-  const long long slots = 152ll * (per_sm > 0 ? per_sm : 1);
+  if (per_sm < 1) per_sm = 1;
   int best = 16;
   double cost = 1e300;
   const int least = sizeof(T) == 8 || (long long)nx * c.ny * c.nz <= (1 << 18) ? least_planes(c) : 16;
   for (int x = least; x <= 40; ++x) {
     const long long blocks = (long long)yblocks * ((nx + x - 1) / x);
-    const double t = (double)((blocks + slots - 1) / slots) * (x + 1.5);
+    const long long sm_blocks = (blocks + 151) / 152, waves = (sm_blocks + per_sm - 1) / per_sm;
+    const double t = sizeof(T) == 8 ? (x + 0.7) * std::max((sm_blocks + 0.5) * warps, 5.0 * waves)
+                                    : (double)((blocks + 152ll * per_sm - 1) / (152ll * per_sm)) * (x + 1.5);
     if (t < cost) {
       cost = t;
       best = x;
@@ -2222,7 +2237,7 @@ void launch_rhs(const Consts& c, const Fields<T>& f, int cur, cudaStream_t s) {
       if (!XR) {
         int per_sm = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_rhs_vec<T>, threads, sh);
-        XR = rhs_wave_planes<T>(c, c.ny / RV::TJ, per_sm);
+        XR = rhs_wave_planes<T>(c, c.ny / RV::TJ, per_sm, threads / 32);
       }
       k_rhs_vec<T><<<dim3(c.ny / RV::TJ, (c.nx + XR - 1) / XR), threads, sh, s>>>(
           c, f.prm, f.u[cur], f.v[cur], f.w[cur], f.p, f.n[0], f.n[1], f.n[2], f.d[0], f.d[1],
@@ -2234,7 +2249,7 @@ void launch_rhs(const Consts& c, const Fields<T>& f, int cur, cudaStream_t s) {
   const size_t stage = rhs_stage_bytes<T>(c, TJR);
   const int rs = (int)std::min<size_t>(std::min(RSTAGES_MAX, c.rhs_stages), (size_t)(210 * 1024) / stage);
   if (rs >= 4 && c.ny % TJR == 0 && (c.nz * sizeof(T)) % 16 == 0) {
-    const int XR = c.rhs_planes ? c.rhs_planes : rhs_wave_planes<T>(c, c.ny / TJR, 1);
+    const int XR = c.rhs_planes ? c.rhs_planes : rhs_wave_planes<T>(c, c.ny / TJR, 1, RTHREADS / 32);
     k_rhs_pipe<T, TJR><<<dim3(c.ny / TJR, (c.nx + XR - 1) / XR), RTHREADS, rs * stage, s>>>(
         c, f.prm, f.u[cur], f.v[cur], f.w[cur], f.p, f.n[0], f.n[1], f.n[2], f.d[0], f.d[1],
         f.d[2], XR, rs, inflow_cur_v(c, f), inflow_cur_w(c, f));
@@ -2359,9 +2374,11 @@ bool launch_af_yz(const Consts& c, const Fields<T>& f, int cur, cudaStream_t s) 
   constexpr int J = YZRows<T>::J;
   if (c.ny % J != 0) return false;
   const dim3 grid(c.ny / J, c.nx, 3);
+  const T* tab;
+  if constexpr (sizeof(T) == 8) tab = (const T*)f.taps + yz_table(c); else tab = (const T*)f.tapsf + yz_table(c);
 #define YZ_CASE(EE)                                                                               \
   case 32 * EE:                                                                                   \
-    k_af_yz<T, EE><<<grid, YZ_THREADS, 0, s>>>(c, f.prm, f.e[0], f.e[1], f.e[2], f.u[cur],       \
+    k_af_yz<T, EE><<<grid, YZ_THREADS, 0, s>>>(c, f.prm, tab, f.e[0], f.e[1], f.e[2], f.u[cur],  \
                                               f.v[cur], f.w[cur]);                               \
     return true;
   switch (c.nz) {
@@ -2385,8 +2402,10 @@ void launch_af(const Consts& c, const Fields<T>& f, int cur, cudaStream_t s) {
 template <class T>
 void launch_div(const Consts& c, const Fields<T>& f, int cur, bool initial, cudaStream_t s) {
   if (const RunShape r = run_shape<T>(c, c.nx, 4); r.rows) {
+    const T* tab;
+    if constexpr (sizeof(T) == 8) tab = (const T*)f.taps + yz_table(c); else tab = (const T*)f.tapsf + yz_table(c);
     k_div_vec<T><<<dim3(c.ny / r.rows, (c.nx + r.xch - 1) / r.xch), r.threads, 0, s>>>(
-        c, f.prm, f.u[cur], f.v[cur], f.w[cur], f.phi, initial ? 1 : 0, r.xch);
+        c, f.prm, tab, f.u[cur], f.v[cur], f.w[cur], f.phi, initial ? 1 : 0, r.xch);
     return;
   }
   k_div<T><<<grid3(c, c.nx), dim3(TK, TJ), 0, s>>>(c, f.prm, f.u[cur], f.v[cur], f.w[cur], f.phi,

@@ -17,7 +17,7 @@ struct Fields {
   T* e[3];                    // second buffer of the implicit line solves
   double* ipt;                // x-factor LU inverse pivots (2 x (nx + 2)), per step
   float* iptf;                // the same in FP32
-  double* taps;               // periodic inverse taps along y (ny), z (nz), then free-space x taps
+  double* taps;               // periodic inverse taps along y (ny), z (nz), free-space x taps, y-z table (40)
   float* tapsf;               // the same in FP32
   T* phi;                     // divergence -> transforms -> pressure correction
   T* ptab;                    // Poisson Thomas inverse pivots per distinct mode
