@@ -37,15 +37,13 @@
 //    (8 channels of a pixel are one core-matrix row), the three z taps again
 //    as start-address shifts of the haloed tile, three accumulators (one per
 //    tap) in tensor memory; blocks of 128 pixels filled by bulk copies from
-//    two threads (one per operand), three stages; CTAs split the pixels,
+//    two warps (one per operand, one copy per channel group), three stages; CTAs split the pixels,
 //    their partials are summed in a fixed order (deterministic training).
 //  * small kernels: input assembly, loss and its gradient, bias gradients,
 //    Adam, weight packing, rollout statistics and emission.
 // Every mbarrier wait is bounded; on expiry the kernel sets the error flag,
 // waits (bounded) for its own tensor-core work, frees its tensor memory and
 // returns.
-#include <cuda.h>
-#include <cudaTypedefs.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -141,15 +139,6 @@ __device__ inline void bulk_g2s_u32(uint32_t dst, const void* src, uint32_t byte
   asm volatile(
       "cp.async.bulk.shared::cta.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "l"(src),
       "r"(bytes), "r"(smem_u32(bar))
-      : "memory");
-}
-
-// bulk copy of the tensor-map box at coordinates (x, y, z) of a 3-D map
-__device__ inline void tma_load_3d(uint32_t dst, const CUtensorMap* map, int x, int y, int z, uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(
-          dst),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar))
       : "memory");
 }
 
@@ -396,16 +385,19 @@ struct WgArgs {
   int* error;
 };
 
-// Two threads fill the stages, one tensor-map box per operand and stage
-// (warp 0: the M operand, all 16 channel groups of the run of pixels; warp 2:
-// the N operand; the shifted one with its halo, which the maps store), warp 1
-// (one thread) issues the MMAs; after the last block all warps read the three
-// accumulators out. Maps: 3-D (8 channels, nz + 2 slots, rows x groups),
-// boxes (8, 128 or 130, groups): the box lands as [group][pixel][8], the
-// MN-major core-matrix strips.
+// Two warps fill the stages (warp 0 the M operand, warp 2 the N operand; the
+// shifted one with its halo, which the maps store): one lane per channel group
+// issues one bulk copy of the group's run of 128 or 130 pixels, 2 KB that are
+// contiguous in the map and land as an MN-major core-matrix strip. Warp 1 (one
+// thread) issues the MMAs; after the last block all warps read the three
+// accumulators out.
+// The copies bound this kernel when a stage came as one tensor-map box of
+// 16-byte rows (8 channels): the copy engine takes about a cycle per row, 4160
+// of them a stage against 1536 cycles of MMAs. At 8 x 256 x 256 pixels:
+// 0.194 ms with the boxes, 0.100 ms (1546 TFLOP/s, 0.81 of the measured bf16
+// burst) with one copy per group.
 template <int NB>
-__global__ void __launch_bounds__(WG_THREADS, 1) k_wgrad(WgArgs g, const __grid_constant__ CUtensorMap map_a,
-                                                        const __grid_constant__ CUtensorMap map_b) {
+__global__ void __launch_bounds__(WG_THREADS, 1) k_wgrad(WgArgs g) {
   using C = WgCfg<NB>;
   extern __shared__ __align__(1024) unsigned char wsm[];
   __shared__ uint64_t full[WG_STAGES], empty[WG_STAGES];
@@ -420,7 +412,6 @@ __global__ void __launch_bounds__(WG_THREADS, 1) k_wgrad(WgArgs g, const __grid_
   const uint32_t sbo_a = g.shift_a ? WG_SBO_H : WG_SBO_P;
   const uint32_t sbo_b = g.shift_a ? WG_SBO_P : WG_SBO_H;
   const uint32_t a_bytes = 16 * sbo_a;
-  const uint32_t rows_a = g.shift_a ? WG_KP + 2 : WG_KP, rows_b = g.shift_a ? WG_KP : WG_KP + 2;
   const uint32_t sbase = smem_u32(wsm);
 
   if (warp == 0) tc_alloc(&tmem_slot, C::TMEM_COLS);
@@ -437,28 +428,30 @@ __global__ void __launch_bounds__(WG_THREADS, 1) k_wgrad(WgArgs g, const __grid_
   const uint32_t tmem = tmem_slot;
   bool ok = true;
 
-  if ((warp == 0 || warp == 2) && lane == 0) {
+  if (warp == 0 || warp == 2) {
     const bool is_a = warp == 0;
+    const int C_in = is_a ? 128 : NB, groups = C_in / 8;
+    const bool halo = is_a == (g.shift_a != 0);
+    const uint32_t run = (halo ? WG_KP + 2 : WG_KP) * 16;
+    const char* src = reinterpret_cast<const char*>(is_a ? g.a : g.b);
     for (int i = 0; i < nkb; ++i) {
       const int s = i % WG_STAGES;
-      if (i >= WG_STAGES) ok = mbar_wait(&empty[s], (uint32_t)((i - WG_STAGES) / WG_STAGES) & 1u) && ok;
+      if (lane == 0) {
+        if (i >= WG_STAGES) ok = mbar_wait(&empty[s], (uint32_t)((i - WG_STAGES) / WG_STAGES) & 1u) && ok;
+        mbar_arrive_expect_tx(&full[s], groups * run);
+      }
+      __syncwarp();
       const int kb = kb0 + i;
       const int rr = kb / per_row, zb = (kb - rr * per_row) * WG_KP;
       const int bb = rr / g.ny, y = rr - bb * g.ny;
       int ys = y + dyi - 1;
       ys += (ys < 0) ? g.ny : 0;
       ys -= (ys >= g.ny) ? g.ny : 0;
-      const int rs = bb * g.ny + ys;
-      const uint32_t sa = sbase + (uint32_t)s * C::STAGE;
-      if (is_a) {
-        mbar_arrive_expect_tx(&full[s], 16 * rows_a * 16);
-        const int ra = g.shift_a ? rs : rr, za = g.shift_a ? zb - 1 : zb;
-        tma_load_3d(sa, &map_a, 0, za + 1, ra * 16, &full[s]);
-      } else {
-        mbar_arrive_expect_tx(&full[s], (NB / 8) * rows_b * 16);
-        const int rb = g.shift_a ? rr : rs, zbb = g.shift_a ? zb : zb - 1;
-        tma_load_3d(sa + a_bytes, &map_b, 0, zbb + 1, rb * (NB / 8), &full[s]);
-      }
+      const size_t row = halo ? (size_t)(bb * g.ny + ys) : (size_t)rr;
+      const uint32_t dst = sbase + (uint32_t)s * C::STAGE + (is_a ? 0u : a_bytes);
+      if (lane < groups)
+        bulk_g2s_u32(dst + (uint32_t)lane * run, src + granule(row, lane, halo ? zb - 1 : zb, C_in, g.nz) * 16, run,
+                     &full[s]);
     }
   } else if (warp == 1) {
     if (lane == 0) {
@@ -1009,8 +1002,8 @@ void launch_conv(const ConvArgs& a, cudaStream_t s) {
 }
 
 template <int NB>
-void launch_wgrad(const WgArgs& a, const CUtensorMap& ma, const CUtensorMap& mb, cudaStream_t s) {
-  k_wgrad<NB><<<dim3(a.chunks, 3), WG_THREADS, WgCfg<NB>::SMEM, s>>>(a, ma, mb);
+void launch_wgrad(const WgArgs& a, cudaStream_t s) {
+  k_wgrad<NB><<<dim3(a.chunks, 3), WG_THREADS, WgCfg<NB>::SMEM, s>>>(a);
 }
 
 constexpr int WIDTH = 128;     // channels of the residual stream
@@ -1064,9 +1057,6 @@ struct ibm_gen {
   unsigned long long noise_seed = 0;
   int* error = nullptr;
   std::vector<void*> allocs;
-  // tensor maps of the bfloat16 maps: per base address, boxes of 128 and 130 pixels
-  std::vector<const void*> map_base;
-  std::vector<CUtensorMap> map_box;   // 2 per base: [128-pixel box, 130-pixel box]
 };
 
 namespace {
@@ -1086,41 +1076,6 @@ bool dalloc(ibm_gen* g, T** p, size_t n) {
 
 bf16* act_map(ibm_gen* g, int l) {
   return g->act + (size_t)l * ibm::map_elems((size_t)g->batch * g->ny, ibm::WIDTH, g->nz);
-}
-
-// 3-D tensor maps over a C-channel granule map: (8 channels, nz + 2 slots,
-// rows x C/8 groups), boxes (8, 128 or 130 pixels, C/8 groups)
-bool add_maps(ibm_gen* g, const bf16* base, int C) {
-  static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
-  if (!encode) {
-    void* fn = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) !=
-            cudaSuccess || q != cudaDriverEntryPointSuccess || !fn)
-      return false;
-    encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
-  }
-  const cuuint64_t rows = (cuuint64_t)g->batch * g->ny;
-  const cuuint64_t dims[3] = {8, (cuuint64_t)g->nz + 2, rows * (C / 8)};
-  const cuuint64_t strides[2] = {16, ((cuuint64_t)g->nz + 2) * 16};
-  const cuuint32_t estr[3] = {1, 1, 1};
-  for (int halo = 0; halo < 2; ++halo) {
-    const cuuint32_t box[3] = {8, (cuuint32_t)(ibm::WG_KP + 2 * halo), (cuuint32_t)(C / 8)};
-    CUtensorMap m;
-    if (encode(&m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<bf16*>(base), dims, strides, box, estr,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-      return false;
-    g->map_box.push_back(m);
-  }
-  g->map_base.push_back(base);
-  return true;
-}
-
-const CUtensorMap& tmap(const ibm_gen* g, const bf16* base, bool halo) {
-  size_t i = 0;
-  while (i + 1 < g->map_base.size() && g->map_base[i] != base) ++i;
-  return g->map_box[2 * i + (halo ? 1 : 0)];
 }
 
 int check_error(ibm_gen* g) {
@@ -1168,9 +1123,7 @@ void wgrad(ibm_gen* g, const bf16* a, const bf16* b, int nb, int shift_a, int tr
   WgArgs w{};
   w.a = a; w.b = b; w.shift_a = shift_a; w.ny = g->ny; w.nz = g->nz; w.rows = rows;
   w.chunks = WG_CHUNKS; w.part = g->part; w.error = g->error;
-  const CUtensorMap& ma = tmap(g, a, shift_a != 0);
-  const CUtensorMap& mb = tmap(g, b, shift_a == 0);
-  if (nb == WIDTH) launch_wgrad<WIDTH>(w, ma, mb, g->stream); else launch_wgrad<16>(w, ma, mb, g->stream);
+  if (nb == WIDTH) launch_wgrad<WIDTH>(w, g->stream); else launch_wgrad<16>(w, g->stream);
   const int n = 9 * L.O * L.C;
   k_wgrad_reduce<<<(n + 255) / 256, 256, 0, g->stream>>>(g->part, WG_CHUNKS, nb, trans, L.O, L.C, g->gw + L.woff);
 }
@@ -1325,13 +1278,6 @@ int ibm_gen_create(const ibm_gen_config* cfg, ibm_gen** out) {
   cudaMemsetAsync(g->m, 0, g->np * sizeof(float), g->stream);
   cudaMemsetAsync(g->v, 0, g->np * sizeof(float), g->stream);
   cudaMemsetAsync(g->x, 0, map_elems(rows, CIN_PAD, g->nz) * sizeof(bf16), g->stream);
-  bool maps = add_maps(g, g->x, CIN_PAD) && add_maps(g, g->gd16, COUT_PAD) && add_maps(g, g->g16[0], WIDTH) &&
-              add_maps(g, g->g16[1], WIDTH);
-  for (int l = 0; l <= g->blocks && maps; ++l) maps = add_maps(g, act_map(g, l), WIDTH);
-  if (!maps) {
-    ibm_gen_destroy(g);
-    return IBM_ECUDA;
-  }
   cudaMemsetAsync(g->hist[0], 0, g->P * 3 * sizeof(float), g->stream);
   cudaMemsetAsync(g->hist[1], 0, g->P * 3 * sizeof(float), g->stream);
   cudaMemsetAsync(g->error, 0, sizeof(int), g->stream);
