@@ -1355,6 +1355,7 @@ __global__ void __launch_bounds__(YZ_THREADS)
 k_af_yz(Consts c, const Params* __restrict__ prm, const T* __restrict__ tab, const T* __restrict__ e0,
         const T* __restrict__ e1, const T* __restrict__ e2, T* __restrict__ u,
         T* __restrict__ v, T* __restrict__ w) {
+  grid_ready(prm, tab, e0, e1, e2, u, v, w);
   constexpr int NZ = 32 * E;
   constexpr int LDP = NZ + NZ / 32;
   constexpr int J = YZRows<T>::J;
@@ -1870,6 +1871,7 @@ k_project_vec(Consts c, const Params* __restrict__ prm, const T* __restrict__ ua
               const T* __restrict__ va, const T* __restrict__ wa, T* __restrict__ ub,
               T* __restrict__ vb, T* __restrict__ wb, const T* __restrict__ phi, const void* __restrict__ phi_b,
               T* __restrict__ p, double* __restrict__ partial, int initial, int xch) {
+  grid_ready(prm, ua, va, wa, ub, vb, wb, phi, phi_b, p, partial);
   constexpr int E = RunTile<T>::E;
   const T* pb = static_cast<const T*>(phi_b);
   const __nv_bfloat16* pb16 = static_cast<const __nv_bfloat16*>(phi_b);
@@ -2009,6 +2011,7 @@ k_project_vec64(Consts c, const Params* __restrict__ prm, const double* __restri
                 const double* __restrict__ wa, double* __restrict__ ub, double* __restrict__ vb, double* __restrict__ wb,
                 const double* __restrict__ phi, double* __restrict__ p, double* __restrict__ partial, int initial,
                 int xch) {
+  grid_ready(prm, ua, va, wa, ub, vb, wb, phi, p, partial);
   using T = double;
   constexpr int E = RunTile<T>::E;
   const int nx = c.nx, ny = c.ny, nz = c.nz;
@@ -2378,7 +2381,7 @@ bool launch_af_yz(const Consts& c, const Fields<T>& f, int cur, cudaStream_t s) 
   if constexpr (sizeof(T) == 8) tab = (const T*)f.taps + yz_table(c); else tab = (const T*)f.tapsf + yz_table(c);
 #define YZ_CASE(EE)                                                                               \
   case 32 * EE:                                                                                   \
-    k_af_yz<T, EE><<<grid, YZ_THREADS, 0, s>>>(c, f.prm, tab, f.e[0], f.e[1], f.e[2], f.u[cur],  \
+    launch_next(k_af_yz<T, EE>, grid, YZ_THREADS, 0, s, c, f.prm, tab, f.e[0], f.e[1], f.e[2], f.u[cur],  \
                                               f.v[cur], f.w[cur]);                               \
     return true;
   switch (c.nz) {
@@ -2423,22 +2426,22 @@ void launch_project(const Consts& c, const Fields<T>& f, int cur, bool initial, 
     const int ini = initial ? 1 : 0;
     if constexpr (sizeof(T) == 4 && RunTile<T>::E == 4) {
       if (phi_b16) {
-        k_project_vec<T, 2><<<grid, r.threads, 0, s>>>(c, f.prm, f.u[cur], f.v[cur], f.w[cur],
+        launch_next(k_project_vec<T, 2>, grid, r.threads, 0, s, c, f.prm, f.u[cur], f.v[cur], f.w[cur],
                                                                 f.u[cur ^ 1], f.v[cur ^ 1], f.w[cur ^ 1],
                                                                 phi_a, phi_b16, f.p, f.partial, ini, r.xch);
         return;
       }
     }
     if constexpr (sizeof(T) == 8) {
-      k_project_vec64<<<grid, r.threads, 0, s>>>(c, f.prm, f.u[cur], f.v[cur], f.w[cur], f.u[cur ^ 1], f.v[cur ^ 1],
+      launch_next(k_project_vec64, grid, r.threads, 0, s, c, f.prm, f.u[cur], f.v[cur], f.w[cur], f.u[cur ^ 1], f.v[cur ^ 1],
                                                  f.w[cur ^ 1], phi_a, f.p, f.partial, ini, r.xch);
     } else {
       if (phi_b)
-        k_project_vec<T, 1><<<grid, r.threads, 0, s>>>(c, f.prm, f.u[cur], f.v[cur], f.w[cur],
+        launch_next(k_project_vec<T, 1>, grid, r.threads, 0, s, c, f.prm, f.u[cur], f.v[cur], f.w[cur],
                                                                 f.u[cur ^ 1], f.v[cur ^ 1], f.w[cur ^ 1],
                                                                 phi_a, phi_b, f.p, f.partial, ini, r.xch);
       else
-        k_project_vec<T, 0><<<grid, r.threads, 0, s>>>(c, f.prm, f.u[cur], f.v[cur], f.w[cur],
+        launch_next(k_project_vec<T, 0>, grid, r.threads, 0, s, c, f.prm, f.u[cur], f.v[cur], f.w[cur],
                                                                 f.u[cur ^ 1], f.v[cur ^ 1], f.w[cur ^ 1],
                                                                 phi_a, nullptr, f.p, f.partial, ini, r.xch);
     }

@@ -463,6 +463,7 @@ __global__ void __launch_bounds__(IB_THREADS)
 k_ib_interp_tiles(Consts c, Params* prm, Markers m, Flag fl, const T* __restrict__ bw,
                   const int* __restrict__ bo, const T* __restrict__ u, const T* __restrict__ v,
                   const T* __restrict__ w) {
+  grid_ready(prm, bw, bo, u, v, w);
   extern __shared__ __align__(16) unsigned char ib_smem[];
   T* box = reinterpret_cast<T*>(ib_smem);
   if (blockIdx.x == 0 && threadIdx.x == 0 && m.nf > 0) {   // hand this step's dt to the structure
@@ -522,6 +523,7 @@ template <class T>
 __global__ void __launch_bounds__(IB_THREADS)
 k_ib_spread_tiles(Consts c, Markers m, Flag fl, const T* __restrict__ bw, const int* __restrict__ bo,
                   T* __restrict__ u, T* __restrict__ v, T* __restrict__ w) {
+  grid_ready(bw, bo, u, v, w);
   extern __shared__ __align__(16) unsigned char ib_smem[];
   T* box = reinterpret_cast<T*>(ib_smem);
   if ((int)blockIdx.x >= m.n_tiles) {
@@ -687,6 +689,7 @@ void ib_set_attributes() {
 // the bars cut, alpha the cell's solid fraction (zero velocity inside)
 template <class T>
 __global__ void k_bar_mask(Markers m, T* __restrict__ u, T* __restrict__ v, T* __restrict__ w) {
+  grid_ready(u, v, w);
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int n0 = m.nbm[0], n1 = n0 + m.nbm[1], n2 = n1 + m.nbm[2];
   if (i >= n2) return;
@@ -698,7 +701,7 @@ template <class T>
 void launch_ib(const Consts& c, const Fields<T>& f, const Markers& m, const Flag& fl, int cur,
                cudaStream_t s) {
   const int nbm = m.nbm[0] + m.nbm[1] + m.nbm[2];
-  if (nbm) k_bar_mask<T><<<(nbm + 255) / 256, 256, 0, s>>>(m, f.u[cur], f.v[cur], f.w[cur]);
+  if (nbm) launch_next(k_bar_mask<T>, (nbm + 255) / 256, 256, 0, s, m, f.u[cur], f.v[cur], f.w[cur]);
   if (m.nm == 0) return;
   if (m.acc) {   // deterministic: fixed-point scatter per marker, then one addition per node
     const int nb = (m.nm + 127) / 128;
@@ -713,9 +716,9 @@ void launch_ib(const Consts& c, const Fields<T>& f, const Markers& m, const Flag
   const int threads = m.n_tiles ? (m.ty * m.tz < 256 ? IB_THREADS / 2 : IB_THREADS) : FLAG_ITEMS;
   const size_t smem = m.n_tiles ? ib_tile_smem(m, sizeof(T)) : 0;
   const T* bw = reinterpret_cast<const T*>(m.bar_w);
-  k_ib_interp_tiles<T><<<nblk, threads, smem, s>>>(c, f.prm, m, fl, bw, m.bar_o, f.u[cur], f.v[cur],
+  launch_next(k_ib_interp_tiles<T>, nblk, threads, smem, s, c, f.prm, m, fl, bw, m.bar_o, f.u[cur], f.v[cur],
                                                       f.w[cur]);
-  k_ib_spread_tiles<T><<<nblk, threads, sizeof(T) == 8 ? 0 : smem, s>>>(c, m, fl, bw, m.bar_o, f.u[cur], f.v[cur], f.w[cur]);
+  launch_next(k_ib_spread_tiles<T>, nblk, threads, sizeof(T) == 8 ? 0 : smem, s, c, m, fl, bw, m.bar_o, f.u[cur], f.v[cur], f.w[cur]);
 }
 
 template void launch_ib<double>(const Consts&, const Fields<double>&, const Markers&, const Flag&,

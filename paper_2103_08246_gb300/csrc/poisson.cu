@@ -302,6 +302,7 @@ __device__ __forceinline__ Sep<T> separate_ends(Cx<T> z0, Cx<T> zh) {
 
 __global__ void __cluster_dims__(R16_CLUSTER, 1, 1) __launch_bounds__(R16_THREADS, 2)
 k_dht2d_r16(const float* in, float* out, const float* __restrict__ twy) {
+  grid_ready(in, out);
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ Cx<float> tw[256];
   Cx<float>* buf = reinterpret_cast<Cx<float>*>(smem_raw);
@@ -399,6 +400,7 @@ constexpr int DHT1_PAIRS = 16;
 // y: columns of a plane (positions nz apart); pairs (c, c + P) of a tile of 2 P columns
 template <class T, int R1, int R2>
 __global__ void __launch_bounds__(256, 2) k_dht1_y(T* __restrict__ data, int nz, int P, const T* __restrict__ twg) {
+  grid_ready(data);
   constexpr int N = R1 * R2;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Cx<T>* S = reinterpret_cast<Cx<T>*>(smem_raw);   // [N][P], wavenumber k1 + R1 k2 at row k1 R2 + k2
@@ -449,6 +451,7 @@ __global__ void __launch_bounds__(256, 2) k_dht1_y(T* __restrict__ data, int nz,
 // z: contiguous lines; pairs (r, r + P) of 2 P consecutive rows
 template <class T, int R1, int R2>
 __global__ void __launch_bounds__(256, 2) k_dht1_z(T* __restrict__ data, int P, const T* __restrict__ twg) {
+  grid_ready(data);
   constexpr int N = R1 * R2;
   constexpr int LD = N + (R2 > 1 ? R1 : 1);   // one slot of padding per R2
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -549,6 +552,7 @@ struct PlaneSize {
 template <int R1Y, int R2Y, int R1Z, int R2Z>
 __global__ void __launch_bounds__((PlaneSize<R1Y, R2Y, R1Z, R2Z>::THREADS), (PlaneSize<R1Y, R2Y, R1Z, R2Z>::THREADS == 512 ? 2 : 1))
 k_dht2d_plane(const float* in, float* out, const float* __restrict__ twy, const float* __restrict__ twz) {
+  grid_ready(in, out);
   using G = PlaneSize<R1Y, R2Y, R1Z, R2Z>;
   using C = Cx<float>;
   constexpr int NY = G::NY, NZ = G::NZ, NZH = G::NZH, LD = G::LD, TH = G::THREADS;
@@ -918,6 +922,7 @@ __device__ __forceinline__ void px_mean00(S* phi, int P, int nx, int lane, unsig
 template <class T>
 __global__ void __launch_bounds__(32) k_poisson_xs(Consts c, const T* __restrict__ tab, const int* __restrict__ conv,
                                                    T* __restrict__ phi, T scale) {
+  grid_ready(tab, phi);
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int P = c.ny * c.nz, nx = c.nx, lane = threadIdx.x;
   const int jk = blockIdx.x * 32 + lane;
@@ -1006,6 +1011,7 @@ __global__ void __launch_bounds__(32) k_poisson_xs(Consts c, const T* __restrict
 template <class T, class S>
 __global__ void __launch_bounds__(128) k_poisson_x(Consts c, const T* __restrict__ tab, const int* __restrict__ conv,
                                                    S* __restrict__ phi, T scale) {
+  grid_ready(tab, phi);
   const int P = c.ny * c.nz;
   const int jk = blockIdx.x * blockDim.x + threadIdx.x;
   if (jk >= P) return;
@@ -1085,7 +1091,7 @@ void launch_dht_y(const Consts& c, const Fields<T>& f, cudaStream_t s) {
         constexpr int R1 = decltype(r1)::value, R2 = decltype(r2)::value;
         const int P = dht1_pairs((long long)c.nx * c.nz / 2, c.nz / 2);
         const size_t sh = (size_t)R1 * R2 * (P + 1) * sizeof(Cx<T>);
-        k_dht1_y<T, R1, R2><<<c.nx * (c.nz / (2 * P)), dht1_threads(P, std::max(R1, R2)), sh, s>>>(f.phi, c.nz, P, f.tw_y);
+        launch_next(k_dht1_y<T, R1, R2>, c.nx * (c.nz / (2 * P)), dht1_threads(P, std::max(R1, R2)), sh, s, f.phi, c.nz, P, f.tw_y);
       }))
     return;
   const int logn = (int)std::lround(std::log2((double)n));
@@ -1103,7 +1109,7 @@ void launch_dht_z(const Consts& c, const Fields<T>& f, cudaStream_t s) {
         constexpr int R1 = decltype(r1)::value, R2 = decltype(r2)::value;
         const int P = dht1_pairs((long long)c.nx * c.ny / 2, c.ny / 2);
         const size_t sh = ((size_t)(R1 * R2 + (R2 > 1 ? R1 : 1)) * P + R1 * R2) * sizeof(Cx<T>);
-        k_dht1_z<T, R1, R2><<<c.nx * (c.ny / (2 * P)), dht1_threads(P, std::max(R1, R2)), sh, s>>>(f.phi, P, f.tw_z);
+        launch_next(k_dht1_z<T, R1, R2>, c.nx * (c.ny / (2 * P)), dht1_threads(P, std::max(R1, R2)), sh, s, f.phi, P, f.tw_z);
       }))
     return;
   const int logn = (int)std::lround(std::log2((double)n));
@@ -1122,10 +1128,10 @@ void launch_poisson_x_on(const Consts& c, const Fields<T>& f, T* buf, cudaStream
   const T scale = (T)(c.h * c.h / ((double)c.ny * c.nz));
   const size_t line = (size_t)c.nx * 32 * sizeof(T);
   if (line <= PXS_MAX && (P + 31) / 32 <= 152 * (int)(227 * 1024 / (line + 1024))) {
-    k_poisson_xs<T><<<(P + 31) / 32, 32, line, s>>>(c, f.ptab, f.pconv, buf, scale);
+    launch_next(k_poisson_xs<T>, (P + 31) / 32, 32, line, s, c, f.ptab, f.pconv, buf, scale);
     return;
   }
-  k_poisson_x<T, T><<<(P + 127) / 128, 128, 0, s>>>(c, f.ptab, f.pconv, buf, scale);
+  launch_next(k_poisson_x<T, T>, (P + 127) / 128, 128, 0, s, c, f.ptab, f.pconv, buf, scale);
 }
 
 // the same on bfloat16 storage (FP32 arithmetic)
@@ -1133,7 +1139,7 @@ void launch_poisson_x_bf16(const Consts& c, const Fields<float>& f, void* buf, c
   const int P = c.ny * c.nz;
   const float scale = (float)(c.h * c.h / ((double)c.ny * c.nz));
   __nv_bfloat16* b = reinterpret_cast<__nv_bfloat16*>(buf);
-  k_poisson_x<float, __nv_bfloat16><<<(P + 127) / 128, 128, 0, s>>>(c, f.ptab, f.pconv, b, scale);
+  launch_next(k_poisson_x<float, __nv_bfloat16>, (P + 127) / 128, 128, 0, s, c, f.ptab, f.pconv, b, scale);
 }
 
 template <class T>
@@ -1148,11 +1154,11 @@ void launch_poisson_x(const Consts& c, const Fields<T>& f, cudaStream_t s) {
 // 256: 2.06 ms in the cluster form, 1.88 here)
 bool launch_dht2d_on(const Consts& c, const Fields<float>& f, const float* in, float* out, cudaStream_t s) {
   if (c.ny == 256 && c.nz == 256) {
-    k_dht2d_r16<<<c.nx * R16_CLUSTER, R16_THREADS, R16_SMEM, s>>>(in, out, f.tw_y);
+    launch_next(k_dht2d_r16, c.nx * R16_CLUSTER, R16_THREADS, R16_SMEM, s, in, out, f.tw_y);
     return true;
   }
   return with_plane(c.ny, c.nz, [&](auto g, auto kernel) {
-    kernel<<<c.nx, decltype(g)::THREADS, decltype(g)::SMEM, s>>>(in, out, f.tw_y, f.tw_z);
+    launch_next(kernel, c.nx, decltype(g)::THREADS, decltype(g)::SMEM, s, in, out, f.tw_y, f.tw_z);
   });
 }
 template <class T>
@@ -1165,7 +1171,7 @@ bool launch_dht2d(const Consts& c, const Fields<T>& f, cudaStream_t s) {
 // (the generator's spectral relaxation); tw: the 256-point twiddles
 bool dht2d_planes_fp32(const float* in, float* out, int nplanes, const float* tw, cudaStream_t s) {
   if (nplanes <= 0) return true;
-  k_dht2d_r16<<<nplanes * R16_CLUSTER, R16_THREADS, R16_SMEM, s>>>(in, out, tw);
+  launch_next(k_dht2d_r16, nplanes * R16_CLUSTER, R16_THREADS, R16_SMEM, s, in, out, tw);
   return cudaGetLastError() == cudaSuccess;
 }
 
