@@ -777,7 +777,7 @@ int init_state(ibm_state* s, const ibm_options* o, const FlagGeom& fg,
   ib_set_attributes();
   launch_ib_setup<T>(c, f, m, st);   // the bar markers' weights and box indices, once
   CK(cudaGetLastError());
-  poisson_set_attributes();
+  poisson_set_attributes(c.ny, c.nz);
   fluid_set_attributes();
   mixed_set_attributes();
   if (s->precision == IBM_MIXED) {

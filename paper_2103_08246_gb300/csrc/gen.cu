@@ -62,7 +62,7 @@
 namespace ibm {
 // the FP32 2-D Hartley transform of 256 x 256 planes (poisson.cu)
 bool dht2d_planes_fp32(const float* in, float* out, int nplanes, const float* tw, cudaStream_t s);
-void poisson_set_attributes();
+void poisson_set_attributes(int ny, int nz);
 }  // namespace ibm
 
 namespace ibm {
@@ -1519,7 +1519,7 @@ int ibm_gen_set_spectrum(ibm_gen* g, const double* power, double lambda) {
     if (!dalloc(g, &g->spec, 3 * P) || !dalloc(g, &g->sbuf[0], 3 * P) || !dalloc(g, &g->sbuf[1], 3 * P) ||
         !dalloc(g, &g->twz, 256))
       return IBM_ENOMEM;
-    ibm::poisson_set_attributes();
+    ibm::poisson_set_attributes(256, 256);
   }
   std::vector<float> sp(3 * P), tw(256);
   for (size_t i = 0; i < 3 * P; ++i) sp[i] = (float)power[i];

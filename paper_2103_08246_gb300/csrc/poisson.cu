@@ -1213,16 +1213,16 @@ template void launch_poisson<float>(const Consts&, const Fields<float>&, cudaStr
 template void launch_poisson_table<double>(const Consts&, const Fields<double>&, cudaStream_t);
 template void launch_poisson_table<float>(const Consts&, const Fields<float>&, cudaStream_t);
 
-// opt in to large dynamic shared memory for the transform kernels
-void poisson_set_attributes() {
+// opt in to large dynamic shared memory for the transform kernels of ny x nz
+// planes (setting it for every size loads every kernel: 0.4 ms of a process's first create)
+void poisson_set_attributes(int ny, int nz) {
   cudaFuncSetAttribute(k_dht2d_r16, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)R16_SMEM);
   cudaFuncSetAttribute(k_poisson_xs<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PXS_MAX);
   cudaFuncSetAttribute(k_poisson_xs<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PXS_MAX);
-  for (int n = 4; n <= 256; n *= 2) {
-    for (int m = 4; m <= 256; m *= 2)
-      with_plane(n, m, [](auto g, auto kernel) {
-        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)decltype(g)::SMEM);
-      });
+  with_plane(ny, nz, [](auto g, auto kernel) {
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)decltype(g)::SMEM);
+  });
+  for (int n : {ny, nz})
     with_radices(n, [](auto r1, auto r2) {
       constexpr int R1 = decltype(r1)::value, R2 = decltype(r2)::value;
       cudaFuncSetAttribute(k_dht1_y<double, R1, R2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
@@ -1230,7 +1230,6 @@ void poisson_set_attributes() {
       cudaFuncSetAttribute(k_dht1_y<float, R1, R2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
       cudaFuncSetAttribute(k_dht1_z<float, R1, R2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
     });
-  }
   cudaFuncSetAttribute(k_dht<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
   cudaFuncSetAttribute(k_dht<double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
   cudaFuncSetAttribute(k_dht<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);

@@ -185,7 +185,7 @@ template <class T> void launch_poisson_x(const Consts& c, const Fields<T>& f, cu
 template <class T> void launch_poisson_x_on(const Consts& c, const Fields<T>& f, T* buf, cudaStream_t s);
 void launch_poisson_x_bf16(const Consts& c, const Fields<float>& f, void* buf, cudaStream_t s);
 template <class T> void launch_poisson_table(const Consts& c, const Fields<T>& f, cudaStream_t s);
-void poisson_set_attributes();
+void poisson_set_attributes(int ny, int nz);
 
 // ---- mixed.cu
 // leaves phi = e[1] + e[2] (predictor + correction; the projection sums them)
