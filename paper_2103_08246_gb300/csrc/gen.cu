@@ -1580,6 +1580,7 @@ int ibm_gen_time(ibm_gen* g, int what, int nrep, double* ms) {
         break;
       }
       case 4:
+        cudaEventRecord(g->ev_part[0], g->stream);
         wgrad(g, g->g16[0], act_map(g, 0), WIDTH, 0, rows, 0);
         wgrad_sum(g, WIDTH, 0, g->layers[1], 0);
         side_joins(g);
