@@ -73,12 +73,12 @@ METHOD_PASSES = {"fp32": 57, "mixed": 65}
 # (profiles/launches_production_fp32.md, launches_production_mixed.md);
 # valid for the kernels of those captures and to be refreshed whenever one
 # of them changes.
-_TRAFFIC_COMMON = {"rhs": 1743.1e6, "af_yz": 1156.6e6, "af_x": 752.3e6, "mass_div": 519.2e6,
-                   "poisson_x": 218.4e6, "ib": 57.9e6}
+_TRAFFIC_COMMON = {"rhs": 1720.8e6, "af_yz": 1158.9e6, "af_x": 754.0e6, "mass_div": 513.1e6,
+                   "poisson_x": 218.0e6, "ib": 57.9e6}
 TRAFFIC_BYTES = {
-    "fp32": dict(_TRAFFIC_COMMON, dht2d=209.9e6, project=1181.3e6),
-    "mixed": dict(_TRAFFIC_COMMON, dht2d=212.3e6, tc_bf16=84.6e6, residual=317.6e6, poisson_x16=78.2e6,
-                  project=1258.4e6),
+    "fp32": dict(_TRAFFIC_COMMON, dht2d=209.8e6, project=1181.1e6),
+    "mixed": dict(_TRAFFIC_COMMON, dht2d=212.3e6, tc_bf16=84.2e6, residual=317.7e6, poisson_x16=78.0e6,
+                  project=1261.8e6),
 }
 # the mixed path's projection reads the solve's two parts (FP32 predictor,
 # bfloat16 correction): half a pass more than FIELD_PASSES["project"]
@@ -86,10 +86,10 @@ MIXED_PASSES = {"project": 9.5}
 # FP64 path: the explicit stage's FP64 instructions per cell (DFMA + DMUL +
 # DADD, from an ncu count of k_rhs_vec<double>) and the FP64 issue rate of
 # GB300 (2 per clock per SM): the FP64 step is bound by that pipe.
-FP64_RHS_INST_PER_CELL = 86.2
+FP64_RHS_INST_PER_CELL = 75.9
 # DRAM bytes of one residual-block convolution of the generator (8 x 256 x 256
 # pixels, 128 -> 128 channels) from an ncu capture of the current kernel
-GEN_CONV_TRAFFIC_BYTES = 757.4e6
+GEN_CONV_TRAFFIC_BYTES = 756.3e6
 FP64_INST_PER_CLK_SM = 2
 N_SMS = 152
 CLOCK_WINDOW_S = 0.6   # each leg's clock record spans at least this long
@@ -497,10 +497,10 @@ def stage_roofline(wl, precision, peak_gbs, peak_kind):
                       "alg_bytes_per_launch": nbytes, "achieved_gbs": gbs, "frac": gbs / peak_gbs,
                       "traffic": TRAFFIC_BYTES[key].get(k)}
     kernels["ib"]["nodes_touched"] = ib_nodes
-    # the FP64 flag update (side stream, overlapped with the pressure solve);
+    # the flag update (side stream, overlapped with the pressure solve);
     # its cost scales with the sub-step count of this state's time step
     kernels["flag"] = {"ms_per_launch": stages["flag"], "launches_per_step": 1, "sub_steps": n_sub,
-                       "bound": "fp64 pipe and cluster barriers", "overlapped": True}
+                       "bound": "chain of sub-steps (shared-memory gathers, cluster barriers)", "overlapped": True}
     dom = max((k for k in kernels if k not in ("ib", "flag")), key=lambda k: per_step[k])
     d = kernels[dom]
     roof = {"kernel": dom, "bound": "hbm", "achieved": d["achieved_gbs"], "peak": peak_gbs,

@@ -56,10 +56,10 @@ extern "C" {
 
 /* arithmetic of the fluid fields */
 #define IBM_FP64  0        /* everything in FP64                               */
-#define IBM_FP32  1        /* fluid fields and kernels in FP32; flag, sums FP64 */
-#define IBM_MIXED 2        /* FP32 fields; Poisson transforms as split-TF32 tensor-core
-                              GEMMs (FP32 accumulation) + one refinement sweep on a
-                              residual evaluated in double-single (FP64-class)
+#define IBM_FP32  1        /* fluid fields and kernels in FP32; flag state, sums FP64 */
+#define IBM_MIXED 2        /* FP32 fields; a Poisson solve by FP32 FFTs (tensor-core
+                              GEMMs with mixed_tc_predictor) + one refinement sweep
+                              on a residual evaluated in double-single (FP64-class)
                               arithmetic */
 
 /* stages for ibm_time_stage (Sec. II.B step order) */
