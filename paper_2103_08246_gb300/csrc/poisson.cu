@@ -397,6 +397,13 @@ __device__ __forceinline__ void dft_r(Cx<T> (&x)[R]) {
   else if constexpr (R == 4) dft4_cx(x[0], x[1], x[2], x[3]);
 }
 constexpr int DHT1_PAIRS = 16;
+// the separation's values are twice the transform's. FP64 leaves the factor in
+// (one instruction in 14.4 per value on the pipe that bounds the kernels); the
+// x solve's right-hand side takes it out (poisson_rhs_scale), exactly
+template <class T>
+__device__ __forceinline__ T dht1_norm(T v) {
+  return sizeof(T) == 8 ? v : (T)0.5 * v;
+}
 // y: columns of a plane (positions nz apart); pairs (c, c + P) of a tile of 2 P columns
 template <class T, int R1, int R2>
 __global__ void __launch_bounds__(256, 2) k_dht1_y(T* __restrict__ data, int nz, int P, const T* __restrict__ twg) {
@@ -442,10 +449,10 @@ __global__ void __launch_bounds__(256, 2) k_dht1_y(T* __restrict__ data, int nz,
     const Sep<T> o = k ? separate(zk, zm) : separate_ends(zk, zm);
     T* a = base + (size_t)k * nz + c;
     T* b = base + (size_t)km * nz + c;
-    a[0] = (T)0.5 * o.ak;
-    a[P] = (T)0.5 * o.bk;
-    b[0] = (T)0.5 * o.am;
-    b[P] = (T)0.5 * o.bm;
+    a[0] = dht1_norm<T>(o.ak);
+    a[P] = dht1_norm<T>(o.bk);
+    b[0] = dht1_norm<T>(o.am);
+    b[P] = dht1_norm<T>(o.bm);
   }
 }
 // z: contiguous lines; pairs (r, r + P) of 2 P consecutive rows
@@ -493,10 +500,10 @@ __global__ void __launch_bounds__(256, 2) k_dht1_z(T* __restrict__ data, int P, 
     const Sep<T> o = k ? separate(zk, zm) : separate_ends(zk, zm);
     T* a = base + (size_t)r * N;
     T* b = a + (size_t)P * N;
-    a[k] = (T)0.5 * o.ak;
-    b[k] = (T)0.5 * o.bk;
-    a[km] = (T)0.5 * o.am;
-    b[km] = (T)0.5 * o.bm;
+    a[k] = dht1_norm<T>(o.ak);
+    b[k] = dht1_norm<T>(o.bk);
+    a[km] = dht1_norm<T>(o.am);
+    b[km] = dht1_norm<T>(o.bm);
   }
 }
 // calls f with the radices of an n-point line as integral constants; false beyond 256 points
@@ -1122,10 +1129,20 @@ void launch_dht_z(const Consts& c, const Fields<T>& f, cudaStream_t s) {
 
 constexpr size_t PXS_MAX = 200 * 1024;
 
+// h^2 / (ny nz) for the x solve's right-hand side; in FP64 also 1 / 4 for each
+// direction that k_dht1_y, k_dht1_z transform (there and back, a factor 2 each)
+double poisson_rhs_scale(const Consts& c, bool fp64) {
+  double s = c.h * c.h / ((double)c.ny * c.nz);
+  if (fp64)
+    for (int n : {c.ny, c.nz})
+      if (with_radices(n, [](auto, auto) {})) s *= 0.25;
+  return s;
+}
+
 template <class T>
 void launch_poisson_x_on(const Consts& c, const Fields<T>& f, T* buf, cudaStream_t s) {
   const int P = c.ny * c.nz;
-  const T scale = (T)(c.h * c.h / ((double)c.ny * c.nz));
+  const T scale = (T)poisson_rhs_scale(c, sizeof(T) == 8);
   const size_t line = (size_t)c.nx * 32 * sizeof(T);
   if (line <= PXS_MAX && (P + 31) / 32 <= 152 * (int)(227 * 1024 / (line + 1024))) {
     launch_next(k_poisson_xs<T>, (P + 31) / 32, 32, line, s, c, f.ptab, f.pconv, buf, scale);

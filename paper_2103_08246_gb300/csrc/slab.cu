@@ -289,13 +289,13 @@ void slab_tables(const Consts& c, const SlabDev& sd, cudaStream_t s) {
 
 void slab_local_solve(const Consts& c, const SlabDev& sd, const double* phi, double* send, cudaStream_t s) {
   const int P = c.ny * c.nz;
-  const double scale = c.h * c.h / ((double)c.ny * c.nz);
+  const double scale = poisson_rhs_scale(c, true);
   k_slab_local<<<(P + 127) / 128, 128, 0, s>>>(c, sd, phi, scale, send);
 }
 
 void slab_correct(const Consts& c, const SlabDev& sd, double* phi, const double* gathered, cudaStream_t s) {
   const int P = c.ny * c.nz;
-  const double scale = c.h * c.h / ((double)c.ny * c.nz);
+  const double scale = poisson_rhs_scale(c, true);
   k_slab_correct<<<(P + 127) / 128, 128, 0, s>>>(c, sd, phi, scale, gathered, 1.0 / sd.nx_global);
 }
 

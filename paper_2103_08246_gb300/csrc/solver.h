@@ -181,6 +181,7 @@ template <class T> void launch_stats(const Consts& c, const Fields<T>& f, int cu
 template <class T> void launch_poisson(const Consts& c, const Fields<T>& f, cudaStream_t s);
 template <class T> void launch_dht_y(const Consts& c, const Fields<T>& f, cudaStream_t s);
 template <class T> void launch_dht_z(const Consts& c, const Fields<T>& f, cudaStream_t s);
+double poisson_rhs_scale(const Consts& c, bool fp64);   // poisson.cu: the x solves' factor on transformed data
 template <class T> void launch_poisson_x(const Consts& c, const Fields<T>& f, cudaStream_t s);
 template <class T> void launch_poisson_x_on(const Consts& c, const Fields<T>& f, T* buf, cudaStream_t s);
 void launch_poisson_x_bf16(const Consts& c, const Fields<float>& f, void* buf, cudaStream_t s);
