@@ -351,32 +351,41 @@ __global__ void __launch_bounds__(CV_THREADS, 1) k_conv(ConvArgs g) {
     constexpr int CW = N < 32 ? N : 32;
     constexpr int SPLIT = N >= 64 ? 2 : 1;
     constexpr int HC = N / SPLIT / CW, NCH = (TM / 128) * HC;   // this warp's chunks of a tile
-    // chunk i of this warp's sequence over its tiles: pixel (row, z), column c0
-    auto load = [&](int i, EpiIn<CW>& in) {
-      const int tile = blockIdx.x + (i / NCH) * gridDim.x, q = i % NCH;
-      const int row = tile / tiles_per_row;
-      const int z = (tile - row * tiles_per_row) * TM + (q / HC) * 128 + quarter * 32 + lane;
-      epilogue_load<N, CW>(g, (size_t)row, z, part * (N / SPLIT) + (q % HC) * CW, in);
+    // the loads for chunk q of the tile at pixel (row, z0)
+    auto load = [&](int row, int z0, int q, EpiIn<CW>& in) {
+      epilogue_load<N, CW>(g, (size_t)row, z0 + (q / HC) * 128 + quarter * 32 + lane, part * (N / SPLIT) + (q % HC) * CW, in);
     };
-    const int nch = part < SPLIT ? my_tiles * NCH : 0;
-    EpiIn<CW> cur, nxt;
-    if (nch > 0) load(0, cur);
+    // chunks in two alternate buffers (PAR > 1), or moved from one to the other: at 128
+    // pixels a tile 0.937 -> 0.905 ms for 13 blocks of 8 x 24 x 128 (the moves wait for
+    // the loads), at 256 the moves are the faster form (training step of 8 x 256 x 256
+    // 6.6 against 6.9 ms: fewer registers live)
+    constexpr int PAR = TM == 128 && NCH > 1 ? NCH : 1;
+    int row = blockIdx.x / tiles_per_row, z0 = (blockIdx.x - row * tiles_per_row) * TM;
+    EpiIn<CW> in[2];
+    if (part < SPLIT && my_tiles > 0) load(row, z0, 0, in[0]);
     for (int lt = 0; lt < my_tiles; ++lt) {
-      const int tile = blockIdx.x + lt * gridDim.x;
-      const int row = tile / tiles_per_row, z0 = (tile - row * tiles_per_row) * TM;
+      const int next = blockIdx.x + (lt + 1) * gridDim.x;
+      const int row1 = next / tiles_per_row, z1 = (next - row1 * tiles_per_row) * TM;
       ok = mbar_wait(&tfull[lt & 1], (uint32_t)(lt / 2) & 1u) && ok;
       tc_fence_after();
       const uint32_t dbase = tmem + (uint32_t)((lt & 1) * BUF_COLS);
 #pragma unroll 1
-      for (int q = 0; q < NCH && part < SPLIT; ++q) {
-        const int h = q / HC, c0 = part * (N / SPLIT) + (q % HC) * CW;
-        if (lt * NCH + q + 1 < nch) load(lt * NCH + q + 1, nxt);
-        float v[CW];
-        const uint32_t ta = dbase + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(h * N + c0);
-        if constexpr (CW == 32) tc_ld_x32(ta, v); else tc_ld_x16(ta, v);
-        conv_epilogue<N, CW>(g, (size_t)row, z0 + h * 128 + quarter * 32 + lane, c0, v, cur);
-        cur = nxt;
+      for (int q0 = 0; q0 < NCH && part < SPLIT; q0 += PAR) {
+#pragma unroll
+        for (int par = 0; par < PAR; ++par) {
+          const int q = q0 + par, h = q / HC, c0 = part * (N / SPLIT) + (q % HC) * CW;
+          const bool last = q + 1 == NCH;
+          if (!last || lt + 1 < my_tiles)
+            load(last ? row1 : row, last ? z1 : z0, last ? 0 : q + 1, in[PAR == 1 ? 1 : (par + 1) % 2]);
+          float v[CW];
+          const uint32_t ta = dbase + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(h * N + c0);
+          if constexpr (CW == 32) tc_ld_x32(ta, v); else tc_ld_x16(ta, v);
+          conv_epilogue<N, CW>(g, (size_t)row, z0 + h * 128 + quarter * 32 + lane, c0, v, in[par % 2]);
+        }
+        if constexpr (PAR == 1) in[0] = in[1];
       }
+      row = row1;
+      z0 = z1;
       tc_fence_before();
       mbar_arrive(&tempty[lt & 1]);
     }
