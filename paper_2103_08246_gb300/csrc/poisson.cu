@@ -389,7 +389,8 @@ k_dht2d_r16(const float* in, float* out, const float* __restrict__ twy) {
 // value and direction plus two for the separation, against 18 to 24 of k_dht
 // and of the warp-level 256-point form that was here; the blocks are small, so
 // several share an SM and all SMs get the same number. FP64, y + z: 512 planes of
-// 256 x 256 2.26 -> 1.88 ms, 256 of 128 x 128 0.344 -> 0.230.
+// 256 x 256 2.26 -> 1.88 ms, 256 of 128 x 128 0.344 -> 0.230; 1.75 since the
+// separation leaves its factor of two to the x solve.
 template <class T, int R>
 __device__ __forceinline__ void dft_r(Cx<T> (&x)[R]) {
   if constexpr (R == 16) dft16(x);
@@ -1168,7 +1169,7 @@ void launch_poisson_x(const Consts& c, const Fields<T>& f, cudaStream_t s) {
 // shape, 256 x 256 in clusters, planes that fit shared memory one CTA each. FP64
 // takes the directions one by one: its pipe bounds them either way, and the
 // small blocks of k_dht1_y, k_dht1_z fill the SMs evenly (512 planes of 256 x
-// 256: 2.06 ms in the cluster form, 1.88 here)
+// 256: 2.06 ms in the cluster form, 1.75 here)
 bool launch_dht2d_on(const Consts& c, const Fields<float>& f, const float* in, float* out, cudaStream_t s) {
   if (c.ny == 256 && c.nz == 256) {
     launch_next(k_dht2d_r16, c.nx * R16_CLUSTER, R16_THREADS, R16_SMEM, s, in, out, f.tw_y);
