@@ -1027,18 +1027,20 @@ int num_sms() {
 }
 
 // tiles of 256 pixels when the row allows, else 128; one persistent CTA per SM.
-// Where tiles of 128 all find an SM of their own, they take about half as long
-// as those of 256 on half of the SMs (13 blocks of 24 x 256: 0.799 -> 0.615 ms;
-// 6 of 64 x 256 0.471 -> 0.394). Beyond one wave 256 reads the weights half as often.
+// Tiles of 128 take about half as long each, so they also serve rows of 256
+// where they need one wave of CTAs against one (13 blocks of 24 x 256: 0.799 ->
+// 0.615 ms) or three against two (8 of 2 x 85 x 256 0.854 -> 0.792). They read the
+// weights twice as often, which loses from five against three on (5 of 5 x 64 x
+// 256 0.809 -> 0.831).
 template <int N, int KC>
 void launch_conv(const ConvArgs& a, cudaStream_t s) {
   const int sms = num_sms();
-  if (a.nz % 256 == 0 && a.rows * (a.nz / 128) > sms) {
-    const int tiles = a.rows * (a.nz / 256);
+  const int halves = a.rows * (a.nz / 128), waves = (halves + sms - 1) / sms, waves256 = (halves / 2 + sms - 1) / sms;
+  if (a.nz % 256 == 0 && (waves > 3 || waves >= 2 * waves256)) {
+    const int tiles = halves / 2;
     k_conv<N, KC, 256><<<std::min(tiles, sms), CV_THREADS, ConvCfg<N, KC, 256>::SMEM, s>>>(a);
   } else {
-    const int tiles = a.rows * (a.nz / 128);
-    k_conv<N, KC, 128><<<std::min(tiles, sms), CV_THREADS, ConvCfg<N, KC, 128>::SMEM, s>>>(a);
+    k_conv<N, KC, 128><<<std::min(halves, sms), CV_THREADS, ConvCfg<N, KC, 128>::SMEM, s>>>(a);
   }
 }
 

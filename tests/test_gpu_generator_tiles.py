@@ -16,7 +16,7 @@ BLOCKS, CIN = 2, 6
 
 
 @pytest.mark.parametrize("ny,nz,batch", [(3, 128, 1), (19, 128, 8), (20, 128, 8), (40, 128, 8), (52, 384, 1),
-                                         (3, 256, 1), (76, 256, 1), (77, 256, 1), (160, 256, 1)])
+                                         (3, 256, 1), (76, 256, 1), (77, 256, 1), (160, 256, 1), (57, 256, 4), (114, 512, 1)])
 def test_forward_matches_oracle(ny, nz, batch):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
