@@ -688,7 +688,8 @@ std::vector<float4> lattice_rest(const FlagGeom& g, const ibm_bodies& b, Flag& f
   fl.k_edge[3] = pair(b.stretch / (scale * scale));
   fl.force_scale = scale;
   fl.fix_scale = std::ldexp(scale, 49);
-  for (int q = 0; q < 3; ++q) fl.fix_x0[q] = g.X[q] * fl.fix_scale;
+  // origin: a multiple of 1024 scaled units, exact in FP64
+  for (int q = 0; q < 3; ++q) fl.fix_x0[q] = std::nearbyint(g.X[q] * scale / 1024.0) * 1024.0 * 0x1p49;
   return lat;
 }
 

@@ -161,8 +161,14 @@ __global__ void __launch_bounds__(512) k_flag(Params* __restrict__ prm, Flag fl,
 // FP64. The error of a force against 64 bits is not larger than with
 // rsqrt_nr: that estimate carries up to 5e-14, a double-single operation
 // 2^-47 = 7e-15. Edges are exact: each CTA publishes its positions once per
-// sub-step as 64-bit fixed point relative to the flag's corner (resolution
-// 2^-49 of the lattice spacing), and edges are integer differences.
+// sub-step as 64-bit fixed point (2^49 per scaled unit; the longest spring is
+// 1/2 to 1 unit), and edges are integer differences. The origin is a multiple
+// of 1024 units near the flag's corner, so that subtracting it rounds nothing
+// that the FP64 position held above 2^-49. Positions reach 8192 units from it;
+// the longest lattice with patches has a side of 2176 points, at most a unit
+// apart. Beyond that (a flag that has diverged) they saturate, and a patch that
+// has seen such a position, or one that is not a number, leaves its vertices as
+// NaN.
 //
 // Each CTA keeps its vertices and a halo of two lattice points (the reach of
 // the hinge forces) in shared memory, pulls the halo from its neighbours'
@@ -245,15 +251,25 @@ __device__ __forceinline__ DV cross(DV a, DV b) {
   return {ds_det(a.y, b.z, a.z, b.y), ds_det(a.z, b.x, a.x, b.z), ds_det(a.x, b.y, a.y, b.x)};
 }
 
-// an edge from the difference d of its ends' fixed-point positions (2^49 per
-// scaled unit, |d| < 2^58): the upper part d >> 27 is exact in FP32 for a
-// scaled edge below 4, the lower 27 bits round to 24
+// n 2^k for n < 2^23, without the conversion unit
+template <int K>
+__device__ __forceinline__ float scaled_field(unsigned n) {
+  constexpr unsigned top = (unsigned)(127 + 23 + K) << 23;
+  return __uint_as_float(top | n) - __uint_as_float(top);
+}
+// an edge from the difference of its ends' fixed-point positions (2^49 per
+// scaled unit): upper word, next 23 bits and last 9 bits, each exact in FP32
+// (the upper word for edges below 128 units; it cannot overflow). Every bit
+// that the pair has room for is kept: with the lower bits rounded once to 24
+// the forces' error was three to ten times as large.
 __device__ __forceinline__ DS ds_edge(long long b, long long a) {
   const long long d = b - a;
-  const float h = (float)(int)(d >> 27) * 0x1p-22f;
-  const float l = (float)((int)d & ((1 << 27) - 1)) * 0x1p-49f;
-  return quick2(h, l);
+  const unsigned low = (unsigned)d;
+  const DS s = quick2((float)(int)(d >> 32) * 0x1p-17f, scaled_field<-40>(low >> 9));
+  return {s.h, s.l + scaled_field<-49>(low & 511u)};
 }
+constexpr long long PATCH_LIM = 1ll << 62;   // positions saturate here: differences stay in 64 bits
+constexpr int PATCH_SIDE = 4096;             // points along a side, half of what the positions reach
 constexpr size_t PATCH_SMEM_MAX = 220 * 1024;
 constexpr int PATCH_MAXV = 2;        // vertices per thread
 constexpr int PATCH_HALO = 2;
@@ -304,7 +320,7 @@ __device__ __forceinline__ DS spring_coef(DV d, float4 rest, DS k) {
 
 __global__ void __launch_bounds__(512) k_flag_patch(Params* __restrict__ prm, Flag fl, int force) {
   extern __shared__ __align__(16) unsigned char fp_smem[];
-  __shared__ int n_halo;
+  __shared__ int n_halo, lost;   // lost: a position of the patch or its halo is out of range or NaN
   cg::cluster_group cl = cg::this_cluster();
   if (!force && !prm->flag_pending) return;   // same value for every thread of the cluster
   const int rank = (int)cl.block_rank(), tid = threadIdx.x, nt_ = blockDim.x;
@@ -323,7 +339,7 @@ __global__ void __launch_bounds__(512) k_flag_patch(Params* __restrict__ prm, Fl
   auto vloc = [&](int a, int b) { return (a - a0 + PATCH_HALO) * wv + (b - b0 + PATCH_HALO); };
 
   // halo list: local point, owner and the point in its owner's numbering
-  if (tid == 0) n_halo = 0;
+  if (tid == 0) n_halo = lost = 0;
   __syncthreads();
   const int ha = a1 - a0 + 2 * PATCH_HALO, hb = b1 - b0 + 2 * PATCH_HALO;
   for (int q = tid; q < ha * hb; q += nt_) {
@@ -341,7 +357,6 @@ __global__ void __launch_bounds__(512) k_flag_patch(Params* __restrict__ prm, Fl
            kD = {fl.k_edge[2].x, fl.k_edge[2].y}, ks = {fl.k_edge[3].x, fl.k_edge[3].y};
   const double x0[3] = {fl.fix_x0[0], fl.fix_x0[1], fl.fix_x0[2]};   // scaled origin
   const double fix = fl.fix_scale, back = fl.force_scale;
-  constexpr long long LIM = 1ll << 56;
 
   // this thread's vertices
   const int bw = b1 - b0, nown = (a1 - a0) * bw;
@@ -370,8 +385,9 @@ __global__ void __launch_bounds__(512) k_flag_patch(Params* __restrict__ prm, Fl
       if (own[m] >= 0)
 #pragma unroll
         for (int e = 0; e < 3; ++e) {
-          const long long q = __double2ll_rn(fma(xv[m][e], fix, -x0[e]));
-          X[3 * loc[m] + e] = min(max(q, -LIM), LIM);   // a diverged position stays in the integer range
+          // NaN converts to the lowest integer
+          const long long q = min(max(__double2ll_rn(fma(xv[m][e], fix, -x0[e])), -PATCH_LIM), PATCH_LIM);
+          X[3 * loc[m] + e] = q;
         }
   };
   const int na = a1 - a0, nb = b1 - b0;
@@ -512,13 +528,25 @@ __global__ void __launch_bounds__(512) k_flag_patch(Params* __restrict__ prm, Fl
 #pragma unroll
         for (int e = 0; e < 3; ++e) vv[m][e] = fma(0.5 * hs, acc[m][e], vv[m][e]);
   }
+  // the positions of the last sub-step, those of the halo among them
+  const long long* Xl = X0 + (nsub & 1) * 3 * L.nvert();
+  auto check = [&](int at) {
+    for (int e = 0; e < 3; ++e)
+      if (Xl[3 * at + e] == PATCH_LIM || Xl[3 * at + e] == -PATCH_LIM) lost = 1;
+  };
+  for (int q = tid; q < n_halo; q += nt_) check(halo[q].x);
+#pragma unroll
+  for (int m = 0; m < PATCH_MAXV; ++m)
+    if (own[m] >= 0) check(loc[m]);
+  __syncthreads();
 #pragma unroll
   for (int m = 0; m < PATCH_MAXV; ++m)
     if (own[m] >= 0)
 #pragma unroll
       for (int e = 0; e < 3; ++e) {
-        fl.X[3 * own[m] + e] = xv[m][e];
-        fl.V[3 * own[m] + e] = vv[m][e];
+        const bool keep = !lost || im[m] == 0.0;   // a pinned vertex has not moved
+        fl.X[3 * own[m] + e] = keep ? xv[m][e] : nan("");
+        fl.V[3 * own[m] + e] = keep ? vv[m][e] : nan("");
       }
   cl.sync();   // no CTA leaves while a neighbour may still read its positions
   if (rank == 0 && tid == 0) prm->flag_pending = 0;
@@ -587,10 +615,12 @@ int flag_max_cluster() {
 
 // patches of the lattice for a cluster of up to 16 CTAs: about 64 to 96 vertices
 // each (a smaller patch is mostly halo), none when the largest would not fit in
-// shared memory (lattices beyond 84 x 84 points)
+// shared memory: 84 x 84 points fit, and so do 700 x 9 or 2100 x 2, which the
+// fixed-point positions reach (PATCH_SIDE)
 static PatchSmem patch_of(int ns, int nt, int pr, int pc) { return {(ns + pr - 1) / pr, (nt + pc - 1) / pc}; }
 bool flag_patches(int ns, int nt, int* pr, int* pc) {
   const int most = flag_max_cluster();
+  if (ns > PATCH_SIDE || nt > PATCH_SIDE) return false;
   int n = 1;
   while (2 * n <= most && (long long)ns * nt > 96ll * n) n *= 2;
   int best = 0;
