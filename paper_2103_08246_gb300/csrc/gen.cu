@@ -576,6 +576,7 @@ __global__ void k_wgrad_reduce(const float* __restrict__ part, int chunks, int N
 // narrow for per-element double additions) into entry t of its block's
 // partial row (channel t mod 3); the partials are added in FP64.
 constexpr int COLSUM_BLOCKS = 608;   // 4 per SM
+constexpr int COLSUM_THREADS = 192;  // a multiple of 3
 __global__ void __launch_bounds__(256) k_colsum_part(const float* __restrict__ x, size_t n, double* __restrict__ part) {
   const size_t per = ((n + gridDim.x - 1) / gridDim.x + blockDim.x - 1) / blockDim.x * blockDim.x;
   const size_t lo = (size_t)blockIdx.x * per, hi = min(n, lo + per);
@@ -1055,6 +1056,14 @@ constexpr int COUT_PAD = 16;   // output channels as computed (3 used)
 constexpr int WG_CHUNKS = 50;  // CTAs per tap row of the weight gradients (3 x 50 <= 152 SMs)
 constexpr int SUM_BLOCKS = 152;
 
+// doubles of the partials buffer that a batch of `rows` image rows and `pixels`
+// pixels needs: the most that one of its writers leaves there (bias gradients
+// of a stream and of the output, loss, rollout sums)
+size_t partial_doubles(size_t rows, size_t pixels) {
+  return std::max({rows * WIDTH, (size_t)COLSUM_BLOCKS * COLSUM_THREADS, (pixels + LOSS_THREADS - 1) / LOSS_THREADS,
+                   (size_t)3 * SUM_BLOCKS});
+}
+
 struct Layer {
   int O, C, Op, Cp;        // real and padded output / input channels
   size_t woff, boff;       // offsets of W, b in the flat parameter array
@@ -1184,9 +1193,9 @@ void colsum(ibm_gen* g, const float* x, size_t pixels, int C, float* out) {
     const int rows = (int)(pixels / g->nz);
     ibm::k_colsum_stream<<<rows * (C / 4), 64, 0, g->side>>>(reinterpret_cast<const float4*>(x), g->nz, C, g->dpart);
     ibm::k_colsum_final<<<C, 256, 0, g->side>>>(g->dpart, rows, C, C, out);
-  } else {            // C = 3: 192 threads, one channel each
-    ibm::k_colsum_part<<<ibm::COLSUM_BLOCKS, 192, 0, g->side>>>(x, pixels * C, g->dpart);
-    ibm::k_colsum_final<<<C, 256, 0, g->side>>>(g->dpart, ibm::COLSUM_BLOCKS, 192, C, out);
+  } else {            // C = 3: one channel per thread
+    ibm::k_colsum_part<<<ibm::COLSUM_BLOCKS, ibm::COLSUM_THREADS, 0, g->side>>>(x, pixels * C, g->dpart);
+    ibm::k_colsum_final<<<C, 256, 0, g->side>>>(g->dpart, ibm::COLSUM_BLOCKS, ibm::COLSUM_THREADS, C, out);
   }
 }
 
@@ -1349,7 +1358,7 @@ int ibm_gen_create(const ibm_gen_config* cfg, ibm_gen** out) {
        dalloc(g, &g->delta, BP * 3) && dalloc(g, &g->target, BP * 3) && dalloc(g, &g->gd32, BP * 3) &&
        dalloc(g, &g->part[0], (size_t)3 * WG_CHUNKS * 3 * 128 * WIDTH) &&
        dalloc(g, &g->part[1], (size_t)3 * WG_CHUNKS * 3 * 128 * WIDTH) &&
-       dalloc(g, &g->dpart, (size_t)std::max<size_t>(COLSUM_BLOCKS * 1024, BP / LOSS_THREADS + 1)) &&
+       dalloc(g, &g->dpart, partial_doubles(rows, BP)) &&
        dalloc(g, &g->dscal, 8) && dalloc(g, &g->hist[0], g->P * 3) && dalloc(g, &g->hist[1], g->P * 3) &&
        dalloc(g, &g->qref, g->P * 3) && dalloc(g, &g->error, 1);
   if (!ok) {
