@@ -156,11 +156,13 @@ __global__ void __launch_bounds__(512) k_flag(Params* __restrict__ prm, Flag fl,
 // instructions per clock and SM: about 500 FP64 instructions per lattice cell
 // and sub-step), then its three barriers and the trips through L2 between
 // them. Here the forces are evaluated in double-single arithmetic (an
-// unevaluated FP32 pair, 48 bits) on the FP32 pipe, which issues 64 times as
-// many instructions per clock; positions, velocities and the integration stay
-// FP64. The error of a force against 64 bits is not larger than with
-// rsqrt_nr: that estimate carries up to 5e-14, a double-single operation
-// 2^-47 = 7e-15. Edges are exact: each CTA publishes its positions once per
+// unevaluated FP32 pair, 48 bits; sums and products after Knuth and Dekker) on
+// the FP32 pipe, which issues 64 times as many instructions per clock;
+// positions, velocities and the integration stay FP64. The error of a force
+// against 64 bits is below that of the list form, whose rsqrt_nr carries up to
+// 5e-14: 0.3 to 0.8 of it over lattices of 9 to 2100 points a side, strains to
+// 1e-2 and bending to 0.1 (33 x 33: 5.9e-14 against 1.9e-13 rms), 0.97 where
+// the springs are too weak to count. Edges are exact: each CTA publishes its positions once per
 // sub-step as 64-bit fixed point (2^49 per scaled unit; the longest spring is
 // 1/2 to 1 unit), and edges are integer differences. The origin is a multiple
 // of 1024 units near the flag's corner, so that subtracting it rounds nothing
@@ -220,15 +222,18 @@ __device__ __forceinline__ DS ds_det(DS a, DS b, DS c, DS d) {
   const DS s = two_sum(p, -q);
   return quick2(s.h, s.l + (pe - qe));
 }
-// 1 / sqrt(x) from the FP32 estimate: with r = 1 - x y0^2 (|r| < 2^-21, its
-// leading difference exact), y0 (1 + r / 2 + 3 r^2 / 8)
+// 1 / sqrt(x) from the FP32 estimate: with r = 1 - x y0^2 (|r| < 2^-21) in two
+// parts, r1 the exact leading difference and r2 the rest,
+// y0 (1 + r / 2 + 3 r^2 / 8); r in one part rounds at 2^-46
 __device__ __forceinline__ DS ds_rsqrt(DS x) {
   const float y = rsqrtf(x.h);
   const float p = __fmul_rn(x.h, y);
   const float pl = fmaf(x.l, y, fmaf(x.h, y, -p));
   const float q = __fmul_rn(p, y);
-  const float r = __fsub_rn(__fsub_rn(1.0f, q), fmaf(p, y, -q)) - pl * y;
-  return quick2(y, y * (r * fmaf(0.375f, r, 0.5f)));
+  const float r1 = __fsub_rn(1.0f, q), r2 = -fmaf(pl, y, fmaf(p, y, -q)), r = r1 + r2;
+  const float t = __fmul_rn(y, 0.5f * r1);
+  const DS s = quick2(y, t);
+  return {s.h, s.l + fmaf(y, fmaf(0.375f * r, r, 0.5f * r2), fmaf(y, 0.5f * r1, -t))};
 }
 // 1 / x
 __device__ __forceinline__ DS ds_rcp(DS x) {
@@ -251,22 +256,17 @@ __device__ __forceinline__ DV cross(DV a, DV b) {
   return {ds_det(a.y, b.z, a.z, b.y), ds_det(a.z, b.x, a.x, b.z), ds_det(a.x, b.y, a.y, b.x)};
 }
 
-// n 2^k for n < 2^23, without the conversion unit
-template <int K>
-__device__ __forceinline__ float scaled_field(unsigned n) {
-  constexpr unsigned top = (unsigned)(127 + 23 + K) << 23;
-  return __uint_as_float(top | n) - __uint_as_float(top);
-}
 // an edge from the difference of its ends' fixed-point positions (2^49 per
 // scaled unit): upper word, next 23 bits and last 9 bits, each exact in FP32
 // (the upper word for edges below 128 units; it cannot overflow). Every bit
 // that the pair has room for is kept: with the lower bits rounded once to 24
-// the forces' error was three to ten times as large.
+// the forces' error was three to ten times as large (33 x 33: 0.1455 ms, 0.149
+// with them).
 __device__ __forceinline__ DS ds_edge(long long b, long long a) {
   const long long d = b - a;
   const unsigned low = (unsigned)d;
-  const DS s = quick2((float)(int)(d >> 32) * 0x1p-17f, scaled_field<-40>(low >> 9));
-  return {s.h, s.l + scaled_field<-49>(low & 511u)};
+  const DS s = quick2((float)(int)(d >> 32) * 0x1p-17f, (float)(low >> 9) * 0x1p-40f);
+  return {s.h, s.l + (float)(low & 511u) * 0x1p-49f};
 }
 constexpr long long PATCH_LIM = 1ll << 62;   // positions saturate here: differences stay in 64 bits
 constexpr int PATCH_SIDE = 4096;             // points along a side, half of what the positions reach
@@ -544,9 +544,8 @@ __global__ void __launch_bounds__(512) k_flag_patch(Params* __restrict__ prm, Fl
     if (own[m] >= 0)
 #pragma unroll
       for (int e = 0; e < 3; ++e) {
-        const bool keep = !lost || im[m] == 0.0;   // a pinned vertex has not moved
-        fl.X[3 * own[m] + e] = keep ? xv[m][e] : nan("");
-        fl.V[3 * own[m] + e] = keep ? vv[m][e] : nan("");
+        fl.X[3 * own[m] + e] = lost ? nan("") : xv[m][e];
+        fl.V[3 * own[m] + e] = lost ? nan("") : vv[m][e];
       }
   cl.sync();   // no CTA leaves while a neighbour may still read its positions
   if (rank == 0 && tid == 0) prm->flag_pending = 0;
