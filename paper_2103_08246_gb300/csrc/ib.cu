@@ -281,14 +281,24 @@ __device__ inline int pos_mod(int a, int n) {
 // 1 - |r| of the outer two is +-r of the middle one, so
 //   s = sqrt(1 - 3 (1/2 - f)^2),  w = ((7/2 - 3 f - s)/6, (1 + s)/3, (1/2 + 3 f - s)/6);
 // 3 square roots per thread instead of 9 (and as many divisions), which bound
-// the FP64 stage: 4225 vertices took 126 + 113 us in 9 blocks of 512.
+// the FP64 stage: 4225 vertices took 126 + 113 us in 9 blocks of 512. A sixth is
+// a product with 1/6 in two parts: with 1/6 rounded to T every weight is too
+// large by the same 3e-8 in FP32, the three directions' sums together by 9e-8,
+// and the speeds of a flag in a uniform stream were up to three times as far
+// from 64 bits (33 x 33: 1.05e-7 against 3.4e-8).
+template <class T>
+__device__ __forceinline__ T sixth(T x) {
+  constexpr T hi = (T)(1.0 / 6.0);
+  constexpr T lo = sizeof(T) == 8 ? (T)0x1.5555555555555p-57 : (T)(1.0 / 6.0 - (double)hi);
+  return fma(x, hi, x * lo);
+}
 template <class T>
 __device__ __forceinline__ void phi3(T f, T w[3]) {
   const T r = (T)0.5 - f;
   const T s = sqrt((T)1 - (T)3 * r * r);
-  w[0] = ((T)3.5 - (T)3 * f - s) * (T)(1.0 / 6.0);
-  w[1] = ((T)1 + s) * (T)(1.0 / 3.0);
-  w[2] = ((T)0.5 + (T)3 * f - s) * (T)(1.0 / 6.0);
+  w[0] = sixth((T)3.5 - (T)3 * f - s);
+  w[1] = sixth((T)2 + (T)2 * s);
+  w[2] = sixth((T)0.5 + (T)3 * f - s);
 }
 // stencil of vertex l on component comp: first node per direction and weights;
 // false for positions that are not finite or absurd (skipped)
