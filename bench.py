@@ -8,8 +8,9 @@ cells, domain 8 x 4 x 4, Re = 200, bar grid (mesh 0.5, width 0.1) at x = 0.5,
 65 x 65 flag hinged at x = 3, CFL 0.3, seeded synthetic initial noise.
 
 Output: one JSON line (rank 0). `value` is steps/s of the mixed-precision
-path (FP32 fields; Poisson transforms as split-TF32 tensor-core GEMMs with a
-refinement sweep on a double-single residual; FP64 flag and global sums)
+path (FP32 fields; an FP32 FFT Poisson solve, refined on a double-single residual
+by a bfloat16 tensor-core solve; flag state and global sums in FP64, the flag's
+forces as FP32 pairs)
 summed over all ranks; each rank runs an independent replica (the path is
 not sharded). Beside it: the FP64 path (the other half of the metric's
 pair) and the FP32 path, each with its own clock record; the roofline of
@@ -835,10 +836,10 @@ def run_ours(args):
             "metric": METRIC, "value": value, "unit": "steps/s", "n_gpus": world,
             "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms,
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
-            "dtype": "mixed: f32 fields, f32 fft predictor, double-single residual, bf16 tensor-core correction, f64 flag",
+            "dtype": "mixed: f32 fields, f32 fft predictor, double-single residual, bf16 tensor-core correction, f64 flag state, f32-pair flag forces",
             "data": "synthetic",
             "config": {"workload": wl.name, "cells": cells,
-                       "precision": "mixed (fp32 fields, fp32 fft predictor, double-single residual, bf16 tcgen05 correction, fp64 flag)",
+                       "precision": "mixed (fp32 fields, fp32 fft predictor, double-single residual, bf16 tcgen05 correction, fp64 flag state, fp32-pair flag forces)",
                        "cfl": wl.cfl, "re": wl.re, "markers": st["n_markers"],
                        "cache": "inputs larger than L2 (each field 134 MB)",
                        "parallelism": f"replicas x{world}"},

@@ -55,23 +55,33 @@ extern "C" {
 #define IBM_EIO       -6   /* checkpoint file could not be written or read    */
 
 /* arithmetic of the fluid fields */
-#define IBM_FP64  0        /* everything in FP64                               */
-#define IBM_FP32  1        /* fluid fields and kernels in FP32; flag state, sums FP64 */
+/* In every precision the flag's state and its integration are FP64; its
+ * internal forces are FP32 pairs (48 bits) on lattices whose patches fit shared
+ * memory (84 x 84 points, 700 x 9) and FP64 on larger ones, the pairs with the
+ * smaller error against 64 bits. */
+#define IBM_FP64  0        /* everything else in FP64                          */
+#define IBM_FP32  1        /* fluid fields and kernels in FP32; sums FP64      */
 #define IBM_MIXED 2        /* FP32 fields; a Poisson solve by FP32 FFTs (tensor-core
                               GEMMs with mixed_tc_predictor) + one refinement sweep
                               on a residual evaluated in double-single (FP64-class)
                               arithmetic */
 
-/* stages for ibm_time_stage (Sec. II.B step order) */
+/* stages for ibm_time_stage (Sec. II.B step order). Not among them: the side
+ * launch beside the explicit stage (the tables of the implicit factors, then the
+ * outflow's increments with the mass fix or, with a prescribed inflow, its mean). */
 #define IBM_STAGE_STEP      -1  /* the whole captured step                   */
 #define IBM_STAGE_RHS        0  /* explicit right-hand side (AB2 + CN half)   */
-#define IBM_STAGE_OUTFLOW    1  /* convective outflow plane                   */
-#define IBM_STAGE_AF_X       2  /* implicit factor along x                    */
+#define IBM_STAGE_OUTFLOW    1  /* convective outflow increments + mass fix in a
+                                   launch of their own, as the step runs them with
+                                   a prescribed inflow (whose new level it takes
+                                   up); without one the side launch does them */
+#define IBM_STAGE_AF_X       2  /* implicit factor along x; advances the outflow
+                                   plane by its increments                    */
 #define IBM_STAGE_AF_Y       3  /* implicit factor along y (periodic), separate */
 #define IBM_STAGE_AF_Z       4  /* implicit factor along z (periodic) + u*, separate */
 #define IBM_STAGE_IB         5  /* marker interpolation + spreading           */
 #define IBM_STAGE_FLAG       6  /* structural sub-steps                       */
-#define IBM_STAGE_MASS_DIV   7  /* mass fix + divergence                      */
+#define IBM_STAGE_MASS_DIV   7  /* divergence, with the mass fix's shift added */
 #define IBM_STAGE_DHT_Y      8  /* transform along y                          */
 #define IBM_STAGE_DHT_Z      9  /* transform along z                          */
 #define IBM_STAGE_POISSON_X 10  /* tridiagonal solves along x                 */

@@ -162,15 +162,15 @@ __global__ void __launch_bounds__(512) k_flag(Params* __restrict__ prm, Flag fl,
 // against 64 bits is below that of the list form, whose rsqrt_nr carries up to
 // 5e-14: 0.3 to 0.8 of it over lattices of 9 to 2100 points a side, strains to
 // 1e-2 and bending to 0.1 (33 x 33: 5.9e-14 against 1.9e-13 rms), 0.97 where
-// the springs are too weak to count. Edges are exact: each CTA publishes its positions once per
-// sub-step as 64-bit fixed point (2^49 per scaled unit; the longest spring is
-// 1/2 to 1 unit), and edges are integer differences. The origin is a multiple
-// of 1024 units near the flag's corner, so that subtracting it rounds nothing
-// that the FP64 position held above 2^-49. Positions reach 8192 units from it;
-// the longest lattice with patches has a side of 2176 points, at most a unit
-// apart. Beyond that (a flag that has diverged) they saturate, and a patch that
-// has seen such a position, or one that is not a number, leaves its vertices as
-// NaN.
+// the springs are too weak to count. Edges are exact: each CTA publishes its
+// positions once per sub-step as 64-bit fixed point (2^49 per scaled unit; the
+// longest spring is 1/2 to 1 unit), and edges are integer differences. The
+// origin is a multiple of 1024 units near the flag's corner, so that subtracting
+// it rounds nothing that the FP64 position held above 2^-49. Positions reach
+// 8192 units from it; the longest lattice with patches has a side of 2176
+// points, at most a unit apart. Beyond that (a flag that has diverged) they
+// saturate, and a patch that has seen such a position, or one that is not a
+// number, leaves its vertices as NaN.
 //
 // Each CTA keeps its vertices and a halo of two lattice points (the reach of
 // the hinge forces) in shared memory, pulls the halo from its neighbours'
@@ -639,8 +639,8 @@ bool flag_patches(int ns, int nt, int* pr, int* pc) {
 
 void launch_flag(Params* prm, const Flag& fl, bool force, cudaStream_t s) {
   if (fl.nv == 0) return;
-  // one CTA per lattice patch where the patches fit (65 x 65: 0.45 -> 0.125 ms
-  // at 8 sub-steps, 33 x 33: 0.63 -> 0.146 ms at 17); the list form otherwise
+  // one CTA per lattice patch where the patches fit (65 x 65: 0.45 -> 0.128 ms
+  // at 8 sub-steps, 33 x 33: 0.64 -> 0.150 ms at 17); the list form otherwise
   if (fl.patch_r) {
     const PatchSmem L = patch_of(fl.ns, fl.nt, fl.patch_r, fl.patch_c);
     const int tasks = 2 * ((L.nnorm() + 31) & ~31);

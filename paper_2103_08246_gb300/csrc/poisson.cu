@@ -925,8 +925,8 @@ __device__ __forceinline__ void px_mean00(S* phi, int P, int nx, int lane, unsig
 // once per chunk of 16 to 32 planes and once per plane of its partial chunks.
 // For grids whose warps fit the SMs together; the low modes, whose pivots
 // converge only after a hundred rows or more, set the time of a small grid.
-// 16,384 modes
-// of 256 planes FP32 0.029 -> 0.0185 ms, 1,024 of 64 FP64 0.025 -> 0.016.
+// 16,384 modes of 256 planes FP32 0.029 -> 0.0185 ms, 1,024 of 64 FP64 0.025 ->
+// 0.016.
 template <class T>
 __global__ void __launch_bounds__(32) k_poisson_xs(Consts c, const T* __restrict__ tab, const int* __restrict__ conv,
                                                    T* __restrict__ phi, T scale) {
